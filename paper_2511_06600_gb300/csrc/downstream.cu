@@ -239,12 +239,28 @@ __device__ __forceinline__ double qval(const T* Q, long long ldq, long long row,
 }
 
 // Centroid rows of the contracted supernodes: one warp per supernode, lanes
-// over columns, members summed in the forming hyperedge's pin order.
+// over columns, members summed in the forming hyperedge's pin order.  Also
+// the FP32 rows mu32 and the column scales that k_seeds bounds distances
+// with: scale[i] = 1/Q_H[i] (0 for columns that take no part), scale[K] = 1
+// when some Q_H lies outside [1e-30, 1e30], where FP32 bounds could overflow
+// or underflow and every distance is formed in FP64.
 template <typename T>
 __global__ void k_centroids(int nc, const int32_t* __restrict__ formed_by,
                             const int* __restrict__ mrow, const int64_t* __restrict__ eptr,
                             const int32_t* __restrict__ pins, const T* __restrict__ Q, long long ldq,
-                            int K, double* __restrict__ mu) {
+                            int K, const double* __restrict__ QH, double* __restrict__ mu,
+                            float* __restrict__ mu32, float* __restrict__ scale) {
+  if (blockIdx.x == 0) {
+    int wide = 0;
+    for (int i = threadIdx.x; i < K; i += blockDim.x) {
+      const double h = QH[i];
+      const bool on = h > 1e-300;
+      wide |= on && !(h >= 1e-30 && h <= 1e30);
+      scale[i] = on ? (float)(1.0 / h) : 0.0f;
+    }
+    wide = __syncthreads_or(wide);
+    if (threadIdx.x == 0) scale[K] = wide ? 1.0f : 0.0f;
+  }
   const int lane = threadIdx.x & 31;
   const int c = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   if (c >= nc) return;
@@ -253,10 +269,13 @@ __global__ void k_centroids(int nc, const int32_t* __restrict__ formed_by,
   const int64_t a = eptr[e], b = eptr[e + 1];
   const double k = (double)(b - a);
   double* row = mu + (size_t)mrow[c] * K;
+  float* row32 = mu32 + (size_t)mrow[c] * K;
   for (int i = lane; i < K; i += 32) {
     double acc = 0.0;
     for (int64_t t = a; t < b; ++t) acc = __dadd_rn(acc, qval(Q, ldq, pins[t], i));
-    row[i] = __ddiv_rn(acc, k);
+    const double x = __ddiv_rn(acc, k);
+    row[i] = x;
+    row32[i] = (float)x;
   }
 }
 
@@ -264,15 +283,32 @@ __global__ void k_centroids(int nc, const int32_t* __restrict__ formed_by,
 // candidate supernode (of a co-pin in a hyperedge containing the vertex) is
 // scored by max over columns of (Q[p,i] - mu_c[i])^2 / Q_H[i]; the smallest
 // score wins, ties to the smallest cluster id.
-template <typename T>
-__global__ void k_seeds(int n, const int32_t* __restrict__ owner, const int32_t* __restrict__ vptr,
-                        const int32_t* __restrict__ vedge, const int32_t* __restrict__ perm,
-                        const int64_t* __restrict__ eptr, const int32_t* __restrict__ pins,
-                        const int32_t* __restrict__ cluster, const int32_t* __restrict__ formed_by,
-                        const int* __restrict__ mrow, const double* __restrict__ mu,
-                        const T* __restrict__ Q, long long ldq, int K,
-                        const double* __restrict__ QH, int32_t* __restrict__ target,
-                        double* __restrict__ dist) {
+//
+// The scores are FP64 (round to nearest), and FP64 division is what bound this
+// kernel (two DFMA per clock and SM): K divisions per candidate pin, 5.68 ms at
+// 210,000 vertices, K = 160; 0.95 ms now.  A candidate is now bounded in FP32 first: with
+// q, m the FP32 roundings of Q[p,i] and mu_c[i], |Q - mu| lies within
+// err = 2^-23 (|q| + |m|) of |q - m|, which gives [lb_i, ub_i] around each
+// column's ratio and [max lb, max ub] around the score (the constants below
+// leave slack for every rounding, underflow included).  A candidate whose lower
+// bound exceeds an earlier candidate's upper bound cannot win; for the others
+// only the columns with ub_i >= max lb can hold the maximum, and only those
+// are formed in FP64: one or two divisions for a few candidates per vertex,
+// with the same result bit for bit.  Columns are held NC per lane, so a
+// candidate costs one FP32 row of gathers.
+template <typename T, int NC>
+__global__ void __launch_bounds__(kThreads)
+    k_seeds(int n, const int32_t* __restrict__ owner, const int32_t* __restrict__ vptr,
+            const int32_t* __restrict__ vedge, const int32_t* __restrict__ perm,
+            const int64_t* __restrict__ eptr, const int32_t* __restrict__ pins,
+            const int32_t* __restrict__ cluster, const int32_t* __restrict__ formed_by,
+            const int* __restrict__ mrow, const double* __restrict__ mu,
+            const float* __restrict__ mu32, const float* __restrict__ scale,
+            const T* __restrict__ Q, long long ldq, int K, const double* __restrict__ QH,
+            int32_t* __restrict__ target, double* __restrict__ dist) {
+  constexpr float kErr = 1.3e-7f;       // > 2^-23
+  constexpr float kSlack = 1e-6f;       // relative, > the products' and scales' roundings
+  constexpr float kTiny = 1e-37f;       // absolute, > what underflow loses
   const int lane = threadIdx.x & 31;
   const int p = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   if (p >= n) return;
@@ -280,30 +316,77 @@ __global__ void k_seeds(int n, const int32_t* __restrict__ owner, const int32_t*
     if (lane == 0) target[p] = -1, dist[p] = 0.0;
     return;
   }
+  const bool wide = scale[K] != 0.0f;
+  float q[NC], sc[NC];
+#pragma unroll
+  for (int t = 0; t < NC; ++t) {
+    const int i = lane + 32 * t;
+    q[t] = i < K ? (float)qval(Q, ldq, p, i) : 0.0f;
+    sc[t] = i < K ? scale[i] : 0.0f;
+  }
   int best = -1;
   double bd = INFINITY;
+  float bound = INFINITY;  // smallest upper bound of a candidate so far
   for (int t = vptr[p]; t < vptr[p + 1]; ++t) {
     const int e = perm[vedge[t]];
-    for (int64_t s = eptr[e]; s < eptr[e + 1]; ++s) {
-      const int u = pins[s];
-      const int c = cluster[u];
-      if (u == p || formed_by[c] < 0) continue;
-      const double* row = mu + (size_t)mrow[c] * K;
-      double d = 0.0;
-      for (int i = lane; i < K; i += 32) {
-        const double qh = QH[i];
-        if (qh > 1e-300) {
-          const double diff = __dsub_rn(qval(Q, ldq, p, i), row[i]);
-          const double r = __ddiv_rn(__dmul_rn(diff, diff), qh);
-          d = r > d ? r : d;
-        }
+    const int64_t b = eptr[e + 1];
+    for (int64_t s0 = eptr[e]; s0 < b; s0 += 32) {
+      int c = -1 - lane, row = 0;
+      if (s0 + lane < b) {
+        const int u = pins[s0 + lane];
+        const int cu = cluster[u];
+        if (u != p && formed_by[cu] >= 0) c = cu, row = mrow[cu];
       }
+      // each supernode once per 32 pins
+      const unsigned peers = __match_any_sync(0xffffffffu, c);
+      unsigned todo = __ballot_sync(0xffffffffu, c >= 0 && lane == __ffs(peers) - 1);
+      while (todo) {
+        const int src = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const int cc = __shfl_sync(0xffffffffu, c, src);
+        const size_t ro = (size_t)__shfl_sync(0xffffffffu, row, src) * K;
+        float m[NC], ub[NC];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const double x = __shfl_xor_sync(0xffffffffu, d, o);
-        d = x > d ? x : d;
+        for (int j = 0; j < NC; ++j) m[j] = lane + 32 * j < K ? mu32[ro + lane + 32 * j] : 0.0f;
+        float lo = 0.0f, hi = 0.0f;
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+          const float d = fabsf(q[j] - m[j]);
+          const float err = kErr * (fabsf(q[j]) + fabsf(m[j]));
+          const float du = d + err, dl = d - err;
+          float u = du * sc[j] * du;
+          u = u * (1.0f + kSlack) + kTiny;
+          if (!(u <= 3.0e38f)) u = INFINITY;  // overflow or NaN: no bound
+          ub[j] = u;
+          hi = fmaxf(hi, u);
+          if (dl > 0.0f) lo = fmaxf(lo, fminf(dl * sc[j] * dl * (1.0f - kSlack), 3.0e38f) - kTiny);
+        }
+        // non-negative floats order as their bits
+        hi = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(hi)));
+        lo = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(lo)));
+        if (wide) lo = 0.0f, hi = INFINITY;
+        if (lo > bound) continue;
+        bound = fminf(bound, hi);
+        double d = 0.0;
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+          const int i = lane + 32 * j;
+          if (i < K && (wide || !(ub[j] < lo))) {
+            const double qh = QH[i];
+            if (qh > 1e-300) {
+              const double diff = __dsub_rn(qval(Q, ldq, p, i), mu[ro + i]);
+              const double r = __ddiv_rn(__dmul_rn(diff, diff), qh);
+              d = r > d ? r : d;
+            }
+          }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const double x = __shfl_xor_sync(0xffffffffu, d, o);
+          d = x > d ? x : d;
+        }
+        if (d < bd || (d == bd && cc < best)) best = cc, bd = d;
       }
-      if (d < bd || (d == bd && c < best)) best = c, bd = d;
     }
   }
   if (lane == 0) {
@@ -539,6 +622,8 @@ struct LevelWs {
   double* eta_next;
   double* eta2;
   double* mu;
+  float* mu32;   // FP32 rows of mu, scale (K + 1): bounds of the seeds' distances
+  float* scale;
   int* minv;
   int* keep;     // m + 1
   int* ne;       // m + 1
@@ -568,6 +653,8 @@ size_t carve_level(void* base, long long n, long long m, int K, LevelWs* w) {
   w->eta_next = c.take<double>(n + 1);
   w->eta2 = c.take<double>(n + 1);
   w->mu = c.take<double>((size_t)(n / 2 + 1) * (K > 0 ? K : 1));
+  w->mu32 = c.take<float>((size_t)(n / 2 + 1) * (K > 0 ? K : 1));
+  w->scale = c.take<float>(K + 1);
   w->minv = c.take<int>(n + 1);
   w->keep = c.take<int>(m + 1);
   w->ne = c.take<int>(m + 1);
@@ -725,12 +812,20 @@ extern "C" hef_status hef_coarsen_level(const hef_incidence* inc, const int64_t*
       using QT = decltype(tag);
       HEF_LAUNCH("k_centroids", st, k_centroids<QT><<<wgrid, kThreads, 0, st>>>(
                                         nn, ws.formed_by, ws.cflag, eptr, pins,
-                                        static_cast<const QT*>(Q), ldq, K, ws.mu));
-      HEF_LAUNCH("k_seeds", st, k_seeds<QT><<<wgrid, kThreads, 0, st>>>(
-                                    nn, out->owner, g.vptr, g.vedge, g.perm, eptr, pins,
-                                    out->cluster, ws.formed_by, ws.cflag, ws.mu,
-                                    static_cast<const QT*>(Q), ldq, K, QH, out->target,
-                                    out->dist));
+                                        static_cast<const QT*>(Q), ldq, K, QH, ws.mu, ws.mu32,
+                                        ws.scale));
+      auto seeds = [&](auto kernel) {
+        HEF_LAUNCH("k_seeds", st, kernel<<<wgrid, kThreads, 0, st>>>(
+                                      nn, out->owner, g.vptr, g.vedge, g.perm, eptr, pins,
+                                      out->cluster, ws.formed_by, ws.cflag, ws.mu, ws.mu32,
+                                      ws.scale, static_cast<const QT*>(Q), ldq, K, QH,
+                                      out->target, out->dist));
+      };
+      // columns per lane: enough registers for K, no more than it needs
+      if (K <= 64) seeds(k_seeds<QT, 2>);
+      else if (K <= 128) seeds(k_seeds<QT, 4>);
+      else if (K <= 256) seeds(k_seeds<QT, 8>);
+      else seeds(k_seeds<QT, 16>);
       return HEF_OK;
     };
     if (dtype == HEF_F64) HEF_PASS(run(double{}));
