@@ -241,4 +241,24 @@ size_t apply_tc_scratch_floats(int K);
 hef_status apply_tc(void* V, bool bf16, long long ldv, long long n, int K, const float* Rinv,
                     int Kp, const float* mu, float* scratch, int* err, cudaStream_t st);
 
+// FP64 Gram and apply by error-free splitting on the tensor cores
+// (ortho_split.cu), for n <= 2^28 rows and K <= 512: exps holds two rows of K
+// exponent fields (the basis as given, then the first pass's output).
+struct SplitWs {
+  long long* hi;
+  long long* lo;
+  int* exps;
+  unsigned char* cols;   // per output column: mean and scale
+  unsigned char* image;  // digits of R^-1
+};
+inline bool split_supported(long long n) { return n <= (1ll << 28); }
+size_t carve_split(Carver& cv, long long n, int K, SplitWs* w);
+hef_status split_col_exps(const double* V, long long ldv, long long n, int K, const SplitWs& w,
+                          cudaStream_t st);
+hef_status gram_split(const double* V, long long ldv, long long n, int K, const int* exps,
+                      const SplitWs& w, double* G, double* c, int* err, cudaStream_t st);
+hef_status apply_split(double* V, long long ldv, long long n, int K, const double* Rinv, int Kp,
+                       const double* mu, const int* exps, int* out_exps, const SplitWs& w, int* err,
+                       cudaStream_t st);
+
 }  // namespace hef

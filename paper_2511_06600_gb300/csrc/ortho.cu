@@ -6,7 +6,9 @@
 // and R2 are upper triangular with positive diagonals, so Q spans the same
 // nested column spaces as V: it is the Gram-Schmidt Q up to rounding.
 //
-// Kernels
+// Kernels (the Gram and the apply run on the tensor cores: ortho_tc.cu for the
+// FP32 and BF16 forms up to K = 511, ortho_split.cu for the FP64 form up to
+// 2^28 rows; k_gram and k_apply serve what those do not take)
 //  k_gram         partial Gram of a row chunk: thread = 8x8 block of the
 //                 upper triangle, FP32 (or FP64) accumulation per chunk, FP64
 //                 partials; k_gram_reduce sums chunks in a fixed order.
@@ -738,6 +740,7 @@ struct OrthoWs {
   int* rank;
   int* flag;
   float* tcs;  // tensor-core apply scratch (FP32 form)
+  SplitWs split;  // tensor-core Gram and apply of the FP64 form
   int nchunk;
   int rows_per_chunk;
   int ngroups;
@@ -757,6 +760,8 @@ size_t carve_ortho(void* base, long long n, int K, int dtype, OrthoWs* w) {
   const size_t KK = (size_t)K * K;
   const size_t esz = dtype == HEF_F64 ? 8 : 4;  // of R^-1 and mu (FP32 for the BF16 basis)
   size_t npart = (size_t)nchunk * npairs * kGB * kGB;
+  const bool split = dtype == HEF_F64 && split_supported(n);
+  if (split) npart = 1;
   if (dtype != HEF_F64 && gram_tc_supported(K)) {
     const size_t tc = gram_tc_part_doubles(n, K);
     if (tc > npart) npart = tc;
@@ -776,6 +781,7 @@ size_t carve_ortho(void* base, long long n, int K, int dtype, OrthoWs* w) {
   w->rank = cv.take<int>(4);
   w->flag = cv.take<int>(4);
   w->tcs = cv.take<float>(dtype != HEF_F64 && apply_tc_supported(K) ? apply_tc_scratch_floats(K) : 1);
+  if (split) carve_split(cv, n, K, &w->split);
   return cv.bytes();
 }
 
@@ -823,12 +829,21 @@ hef_status run_ortho(long long n, int K, T* V, long long ldv, double* R_out, int
   double* Rs[2] = {w.R1, w.R2};
 
   const bool use_tc = sizeof(T) == 4 && gram_tc_supported(K);
+  const bool split = sizeof(T) == 8 && split_supported(n);
   const bool want_R = R_out != nullptr;
   HEF_CHECK_CUDA(cudaMemsetAsync(w.flag, 0, 4 * sizeof(int), st));
+  if (split) {
+    hef_status s = split_col_exps(reinterpret_cast<const double*>(V), ldv, n, K, w.split, st);
+    if (s) return s;
+  }
   for (int pass = 0; pass < 2; ++pass) {
     CholOut o{w.Rinv, w.mu, Rs[pass], w.kept, w.rank, w.flag};
     if (use_tc) {
       hef_status s = gram_tc(V, bf16, ldv, n, K, w.part, w.G, w.c, w.flag + 1, st);
+      if (s) return s;
+    } else if (split) {
+      hef_status s = gram_split(reinterpret_cast<const double*>(V), ldv, n, K,
+                                w.split.exps + pass * K, w.split, w.G, w.c, w.flag + 1, st);
       if (s) return s;
     } else {
       HEF_LAUNCH("k_gram", st, k_gram<T><<<ggrid, kPairs, gram_smem, st>>>(
@@ -872,6 +887,12 @@ hef_status run_ortho(long long n, int K, T* V, long long ldv, double* R_out, int
     if (sizeof(T) == 4 && apply_tc_supported(K)) {
       hef_status s = apply_tc(V, bf16, ldv, n, K, static_cast<const float*>(w.Rinv), Kp,
                               static_cast<const float*>(w.mu), w.tcs, w.flag + 1, st);
+      if (s) return s;
+    } else if (split) {
+      hef_status s = apply_split(reinterpret_cast<double*>(V), ldv, n, K,
+                                 static_cast<const double*>(w.Rinv), Kp,
+                                 static_cast<const double*>(w.mu), w.split.exps + pass * K,
+                                 pass == 0 ? w.split.exps + K : nullptr, w.split, w.flag + 1, st);
       if (s) return s;
     } else {
       HEF_LAUNCH("k_apply", st, k_apply<T><<<agrid, athreads, apply_smem(RB), st>>>(
