@@ -938,7 +938,7 @@ __global__ void __launch_bounds__(kThreads) k_archive_last(IncView g, KView<T> k
 
 // ---------------------------------------------------------------- persistent form
 //
-// All k steps in one cooperative launch of one CTA per SM.  CTA b owns a
+// All k steps in one cooperative launch of at most one CTA per SM.  CTA b owns a
 // contiguous range of vertices and one of hyperedges (internal order),
 // balanced on incidences plus items, and keeps their offsets and index lists
 // in shared memory for all k steps (entries past the capacity are read from
@@ -952,7 +952,13 @@ __global__ void __launch_bounds__(kThreads) k_archive_last(IncView g, KView<T> k
 
 constexpr unsigned int kBarIters = 1u << 21;  // bounded barrier wait (polls of an L2 line: about 1 s)
 constexpr int kCapItems = 4096;               // vertices / hyperedges cached per CTA
-constexpr long long kPersistentMinRows = 32768;  // n + m from which the persistent form runs
+// Rows (n + m) per CTA from which the persistent form takes another CTA, up to
+// one per SM.  Measured from 1 to 152 CTAs: the time of small hypergraphs is
+// flat from about one CTA per 128 rows on (2,048 vertices in FP64, S = 1: 216 us
+// with 32 or 152 CTAs; 8,827 in FP32, S = 4: 302 to 311 us from 64 to 152), and
+// CTAs that gain nothing are left to other streams.  The three launches per
+// step take 377 and 539 us there, so the persistent form runs at every size.
+constexpr long long kPersistentRows = 128;
 constexpr int kCapList = 12288;               // incidences / pins cached per CTA
 constexpr int kPartSlots = 9;                 // reduction slots per start (see part_buffer)
 
@@ -1428,17 +1434,19 @@ hef_status run_krylov_s(const hef_incidence* inc, int k, const double* x0c, cons
   const int grid_n = blocks_for(n);
   const int grid_upd = blocks_for((n + m + upd_rows<T, S>() - 1) / upd_rows<T, S>());
   if (hef_status s0 = krylov_start_s<T, S>(inc, x0c, x0b, kv, st)) return s0;
-  // all steps as one cooperative launch of one CTA per SM (see
+  // all steps as one cooperative launch of at most one CTA per SM (see
   // k_krylov_steps) unless this thread's calls share the GPU with other work
   // (the batched form); if the runtime refuses the grid, three launches per
   // step run instead
-  // (small hypergraphs: the per-step launches are as fast as the barriers)
-  if (persistent && (n + m >= kPersistentMinRows || t_force_oversized)) {
+  if (persistent && n > 0 && m > 0) {
+    const int ctas = t_force_oversized
+                         ? num_sms()
+                         : (int)std::min<long long>(num_sms(), (n + m + kPersistentRows - 1) / kPersistentRows);
     constexpr int NT = pers_threads<T, S>();
     constexpr size_t kSmemLimit = 227 * 1024;  // per-CTA opt-in limit of the sm_100 family
     // list capacities: 1.25 times the average range (the balanced ranges
     // stay within a few per cent of it), at most kCapItems / kCapList
-    const double G = (double)num_sms();
+    const double G = (double)ctas;
     kv.capi = (int)std::min<double>(kCapItems, 1.25 * (double)std::max(n, m) / G + 64.0);
     kv.capl = (int)std::min<double>(kCapList, 1.25 * (double)inc->P / G + 256.0);
     size_t smem = pers_smem<T>(k, S, kv.capi, kv.capl);
@@ -1467,7 +1475,7 @@ hef_status run_krylov_s(const hef_incidence* inc, int k, const double* x0c, cons
       HEF_CHECK_CUDA(cudaMemsetAsync(kv.pcount, 0, flag_words(2 * num_sms()) * sizeof(unsigned int), st));
       // the timeout test launches twice the resident grid as a plain launch,
       // so that the first barrier cannot complete and its bounded wait runs out
-      const int grid = num_sms() * (t_force_oversized ? 2 : 1);
+      const int grid = ctas * (t_force_oversized ? 2 : 1);
       cudaError_t e = cudaSuccess;
       if (t_force_oversized) {
         HEF_LAUNCH("k_krylov_steps", st,
