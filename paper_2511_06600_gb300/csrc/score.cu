@@ -47,6 +47,44 @@ __device__ __forceinline__ float lowest<float>() {
   return -FLT_MAX;
 }
 
+// Running extrema of the staged pass.  FP64 comparisons run at two per clock
+// and SM, a quarter of what integer ones of twice the instructions do, so
+// doubles are compared as order-preserving 64-bit integers; a NaN takes part
+// in neither extremum, as with fmax / fmin.
+template <typename T>
+struct Extrema {
+  T mx, mn;
+  __device__ __forceinline__ void clear() { mx = lowest<T>(), mn = -lowest<T>(); }
+  __device__ __forceinline__ void add(T x) { mx = fmax(mx, x), mn = fmin(mn, x); }
+  __device__ __forceinline__ T spread() const { return mx - mn; }
+  __device__ __forceinline__ void join(int o) {  // with lane ^ o
+    const T ox = __shfl_xor_sync(0xffffffffu, mx, o), on = __shfl_xor_sync(0xffffffffu, mn, o);
+    mx = fmax(mx, ox), mn = fmin(mn, on);
+  }
+};
+template <>
+struct Extrema<double> {
+  long long mx, mn;
+  // the bits of a double with the low 63 inverted when it is negative (its own inverse)
+  static __device__ __forceinline__ long long key(long long b) { return b ^ ((b >> 63) & 0x7fffffffffffffffll); }
+  __device__ __forceinline__ void clear() {
+    mx = key(__double_as_longlong(lowest<double>())), mn = key(__double_as_longlong(-lowest<double>()));
+  }
+  __device__ __forceinline__ void add(double x) {
+    const int hi = __double2hiint(x);
+    const bool number = ((hi & 0x7fffffff) | (__double2loint(x) != 0 ? 1 : 0)) <= 0x7ff00000;
+    const long long k = key(__double_as_longlong(x));
+    if (number) mx = max(mx, k), mn = min(mn, k);
+  }
+  __device__ __forceinline__ double spread() const {
+    return __longlong_as_double(key(mx)) - __longlong_as_double(key(mn));
+  }
+  __device__ __forceinline__ void join(int o) {
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+  }
+};
+
 // An element of Q in the working type T (a BF16 basis widens exactly).
 template <typename T, typename QT>
 __device__ __forceinline__ T qw(QT x) {
@@ -191,20 +229,26 @@ __global__ void __launch_bounds__(256) k_score_big1(IncView g, const QT* __restr
   }
 }
 
-// Q_H from the per-CTA partials (K per CTA, already in red.part) and the large
-// hyperedges' partials, in a fixed order; run by the CTA that completes the
-// grid reduction.
+// This CTA's share of the large hyperedges' partials of column col: rows
+// blockIdx.x, blockIdx.x + gridDim.x, ... (after k_score_big1 has completed).
+// Every CTA adds its own rows to its partial: the last CTA used to add all of
+// them, one dependent load after another, 32 us at the end of a 130 us pass.
+__device__ __forceinline__ double big_share(const double* __restrict__ bpart, int nbpart, int K,
+                                            int col) {
+  double s = 0.0;
+  for (int q = blockIdx.x; q < nbpart; q += gridDim.x) s += bpart[(size_t)q * K + col];
+  return s;
+}
+
+// Q_H from the per-CTA partials (K per CTA, already in red.part) in a fixed
+// order; run by the CTA that completes the grid reduction.
 template <int NC>
-__device__ __forceinline__ void finish_qh(const GridRed& red, int K, const double* __restrict__ bpart,
-                                          int nbpart, double* QH, double* invQH, double* QH_out) {
-  // k_score_big1 (bpart) complete: a no-op unless this pass was launched as
-  // its programmatic dependent
-  pdl_wait();
+__device__ __forceinline__ void finish_qh(const GridRed& red, int K, double* QH, double* invQH,
+                                          double* QH_out) {
   __shared__ double tot[32 * NC];
   if (grid_reduce(red, K, tot)) {
     for (int col = threadIdx.x; col < K; col += blockDim.x) {
-      double s = tot[col];
-      for (int q = 0; q < nbpart; ++q) s += bpart[(size_t)q * K + col];
+      const double s = tot[col];
       QH[col] = s;
       invQH[col] = s > kQhTiny ? 1.0 / s : 0.0;
       if (QH_out) QH_out[col] = s;
@@ -287,47 +331,61 @@ __global__ void __launch_bounds__(256) k_score_pass1(IncView g, const QT* __rest
   for (int col = threadIdx.x; col < K; col += blockDim.x) {
     double s = 0.0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += wred[w][col];
-    red.part[(size_t)blockIdx.x * K + col] = s;
+    red.part[(size_t)blockIdx.x * K + col] = s + big_share(bpart, nbpart, K, col);
   }
-  finish_qh<NC>(red, K, bpart, nbpart, QH, invQH, QH_out);
+  finish_qh<NC>(red, K, QH, invQH, QH_out);
 }
 
 
-// Pass 1 with the pin rows staged in shared memory by bulk asynchronous
-// copies (the same sums as k_score_pass1).  CTA b takes a contiguous range of
-// windows of CSC slots (see kWinSlots) and streams the Q rows of their slots,
-// in slot order, through a ring of `nst` stages of kWinSlots rows (row pitch
-// `pitch` elements, `row_bytes` a multiple of 16): slot t sits in ring row
-// (t - first slot of the range) mod (nst kWinSlots).  Warp 0 produces: it
-// copies window j's rows (G4: four-row tensor-map gathers, tile::gather4 with
-// a box one row high; else one bulk copy per row) once the consumers have
-// released window j - nst
-// (plus the window after the range, whose rows the range's last hyperedges
-// may reach), with the offsets and weights of the hyperedges the window owns
-// (aligned supersets of ceptr[ef..el] and ew[ef..el), when at most
-// kMetaEdges - 8 of them); the pin ids and the window table are loaded a
-// group of kGroupWin windows ahead.  Warps 1..15 consume: for window w, once
-// windows w and w + 1 have landed, each scores the window's hyperedges (first
-// slot in w; at most kBigEdge pins, so they end within w + 1) w, w + 15, ...
-// from shared memory, lanes over columns.  Waits are bounded: on expiry the
-// kernel sets HEF_WAIT_TIMEOUT in `status`, stops, waits (bounded) for the
-// copies it issued and still takes part in the reduction.
+// Pass 1 with the pin rows staged in shared memory by tensor-map gathers (the
+// same sums as k_score_pass1).  The columns are split into `parts` of `pw`
+// (pw * sizeof(T) a multiple of 32, so that four rows are whole 128-byte
+// units); CTA b takes part b mod parts and a contiguous range of windows of CSC
+// slots (see kWinSlots), and streams its columns of the Q rows of their slots,
+// in slot order, through a ring of `nst` stages of kWinSlots rows of pw values:
+// slot t sits in ring row (t - first slot of the range) mod (nst kWinSlots).
+// Warp 0 produces: it copies window j's rows (tile::gather4 with a box one row
+// high; columns past the row's pitch arrive as zeros) once the consumers have
+// released window j - nst (plus the window after the range, whose rows the
+// range's last hyperedges may reach), with the offsets and weights of the
+// hyperedges the window owns (aligned supersets of ceptr[ef..el] and
+// ew[ef..el), when at most kMetaEdges - 8 of them); the pin ids and the window
+// table are loaded a group of kGroupWin windows ahead.  Warps 1..15 consume:
+// for window w, once windows w and w + 1 have landed, the window's hyperedges
+// (first slot in w; at most kBigEdge pins, so they end within w + 1) are scored
+// from shared memory, eight lanes to a hyperedge, in 16-byte chunks: quads of
+// hyperedges (by index, so that consecutive windows keep all warps busy) go to
+// warp (e / 4) mod 15.  Waits are bounded: on expiry the kernel sets
+// HEF_WAIT_TIMEOUT in `status`, stops, waits (bounded) for the copies it issued
+// and still takes part in the reduction.
+//
+// What bounds it: 4 kWinSlots bytes of rows per slot through L2 and the
+// consumers' issue.  Scalar lanes took 20 loads, 20 stores and their addresses
+// per hyperedge and column block; chunks take a quarter.  Parts keep at least
+// four stages in flight where a row is long: with two (K = 384 in FP32, 160 in
+// FP64) every copy was waited for.  Rows whose pitch has no room for the 32-byte
+// rounding, and rows of more than 256 values, used one bulk copy per row.
+// 200,000 nets, K = 160, FP32: 132 -> 117 us (of it 25 us in the last CTA's sum
+// of k_score_big1's partials); 105,001 nets, K = 100: 131 -> 66; 1.3 M nets,
+// K = 384: 2016 -> 1166; FP64, 53,393 nets, K = 160: 309 -> 121 (comparisons).
 static_assert(kBigEdge <= kWinSlots, "a scored hyperedge must end within the next window");
-constexpr int kPinRegs = (kWinSlots + 31) / 32;
 constexpr int kBulkThreads = 512;  // warp 0 produces, warps 1..15 consume
 constexpr int kConsumers = kBulkThreads / 32 - 1;
 constexpr int kGroupWin = 8;    // windows per prefetch group of the producer
 constexpr int kMetaEdges = 128;  // hyperedge offsets / weights staged per window
-constexpr int kFlushWin = 8;     // windows per working-type partial sum of a consumer warp
+constexpr int kFlushWin = 32;    // windows per working-type partial sum of a consumer lane: about ten
+                                 // hyperedges of a group, then four groups, before FP64 takes over
+constexpr int kEdgeLanes = 8;    // lanes per hyperedge
+constexpr int kGroupPins = 12;   // longer hyperedges take the whole warp
+constexpr int kPartChunks = 6;   // 16-byte chunks per lane at most: 768 bytes of a row per part
 constexpr uint32_t kCopyWaitIters = 1u << 20;
 
-template <typename T, int NC, bool G4>
+template <typename T, int C>
 __global__ void __launch_bounds__(kBulkThreads, 1)
-    k_score_pass1_bulk(IncView g, const T* __restrict__ Q, long long ldq, int K, int pitch,
-                       uint32_t row_bytes, int nst, GridRed red, const double* __restrict__ bpart,
-                       int nbpart, double* QH, double* invQH, double* QH_out, T* spread,
-                       int ldsp, const T* __restrict__ ewT, unsigned int* status,
-                       const __grid_constant__ CUtensorMap tmap) {
+    k_score_pass1_bulk(IncView g, int K, int parts, int pw, int nst, GridRed red,
+                       const double* __restrict__ bpart, int nbpart, double* QH, double* invQH,
+                       double* QH_out, T* spread, int ldsp, const T* __restrict__ ewT,
+                       unsigned int* status, const __grid_constant__ CUtensorMap tmap) {
   using namespace umma;
   if (g.status[0]) return;
   extern __shared__ __align__(128) unsigned char stage_raw[];
@@ -343,9 +401,14 @@ __global__ void __launch_bounds__(kBulkThreads, 1)
   volatile int* abort_v = &abort_flag;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const long long nwin = num_windows(g.P);
-  // this CTA's windows [wb, we) and the windows it copies [wb, wc): one
-  // more when it has any, whose first slots its last hyperedges may reach
-  const long long wb = nwin * blockIdx.x / gridDim.x, we = nwin * (blockIdx.x + 1) / gridDim.x;
+  // this CTA's columns [col0, col0 + pcols) and windows [wb, we) (CTAs past
+  // the last whole set of parts have none), and the windows it copies [wb, wc):
+  // one more when it has any, whose first slots its last hyperedges may reach
+  const int part = (int)blockIdx.x % parts, nrange = (int)gridDim.x / parts;
+  const int range = (int)blockIdx.x / parts;
+  const int col0 = part * pw, pcols = min(pw, K - col0);
+  const long long wb = range < nrange ? nwin * range / nrange : nwin;
+  const long long we = range < nrange ? nwin * (range + 1) / nrange : nwin;
   const long long wc = (we > wb && we < nwin) ? we + 1 : we;
   const int ring_rows = nst * kWinSlots;
   if (threadIdx.x == 0) {
@@ -358,9 +421,14 @@ __global__ void __launch_bounds__(kBulkThreads, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  double acc[NC];
+  constexpr int V = 16 / (int)sizeof(T);        // values per chunk
+  constexpr int kGrps = 32 / kEdgeLanes;        // hyperedges per warp at a time
+  constexpr int N = (C * V + kGrps - 1) / kGrps * kGrps;  // column sums of a lane
+  constexpr int NA = N / kGrps;                 // ... kept by each group after a flush
+  double acc[NA];
 #pragma unroll
-  for (int c = 0; c < NC; ++c) acc[c] = 0.0;
+  for (int q = 0; q < NA; ++q) acc[q] = 0.0;
+  const int grp = lane / kEdgeLanes, sub = lane % kEdgeLanes;
   auto fail = [&]() {
     if (lane == 0) {
       *abort_v = 1;
@@ -369,49 +437,36 @@ __global__ void __launch_bounds__(kBulkThreads, 1)
   };
   if (wid == 0) {
     // ---- producer
-    // group buffers of kGroupWin windows from g0: the pin ids (per-row copies:
-    // lane l holds slots l and l + 32 of window g0 + d in pc[d]; gather4: lane
-    // l holds slots 4 (l mod 16) .. + 3 of window g0 + 2 h + l / 16 in pc4[h])
-    // and win_edge[g0 + l] for l <= kGroupWin
-    constexpr int kRegs = G4 ? 1 : kPinRegs;
-    constexpr int kBufs = G4 ? kGroupWin / 2 : kGroupWin;
-    int pc[kBufs][kRegs], pn[kBufs][kRegs];
+    // group buffers of kGroupWin windows from g0: lane l holds the pin ids of
+    // slots 4 (l mod 16) .. + 3 of window g0 + 2 h + l / 16 in pc4[h], and
+    // win_edge[g0 + l] for l <= kGroupWin
+    constexpr int kBufs = kGroupWin / 2;
     int4 pc4[kBufs], pn4[kBufs];
     int wc_e = 0, wn_e = 0;
-    auto load_group = [&](long long g0, int (&pp)[kBufs][kRegs], int4 (&pp4)[kBufs], int& wl) {
-      if constexpr (G4) {
+    auto load_group = [&](long long g0, int4 (&pp4)[kBufs], int& wl) {
 #pragma unroll
-        for (int h = 0; h < kBufs; ++h) {
-          const long long jw = g0 + 2 * h + (lane >> 4);
-          const long long t = jw * kWinSlots + 4 * (lane & 15);
-          pp4[h] = (jw < wc && t < g.P) ? *reinterpret_cast<const int4*>(g.cpins + t)
-                                        : make_int4(0, 0, 0, 0);
-          if (HEF_DEBUG) {
-            // slots past P read as pin 0 of the padded array: only real slots are checked
-            pp4[h].x = t < g.P ? dbg_index(pp4[h].x, g.n, g.status) : pp4[h].x;
-            pp4[h].y = t + 1 < g.P ? dbg_index(pp4[h].y, g.n, g.status) : pp4[h].y;
-            pp4[h].z = t + 2 < g.P ? dbg_index(pp4[h].z, g.n, g.status) : pp4[h].z;
-            pp4[h].w = t + 3 < g.P ? dbg_index(pp4[h].w, g.n, g.status) : pp4[h].w;
-          }
+      for (int h = 0; h < kBufs; ++h) {
+        const long long jw = g0 + 2 * h + (lane >> 4);
+        const long long t = jw * kWinSlots + 4 * (lane & 15);
+        pp4[h] = (jw < wc && t < g.P) ? *reinterpret_cast<const int4*>(g.cpins + t)
+                                      : make_int4(0, 0, 0, 0);
+        if (HEF_DEBUG) {
+          // slots past P read as pin 0 of the padded array: only real slots are checked
+          pp4[h].x = t < g.P ? dbg_index(pp4[h].x, g.n, g.status) : pp4[h].x;
+          pp4[h].y = t + 1 < g.P ? dbg_index(pp4[h].y, g.n, g.status) : pp4[h].y;
+          pp4[h].z = t + 2 < g.P ? dbg_index(pp4[h].z, g.n, g.status) : pp4[h].z;
+          pp4[h].w = t + 3 < g.P ? dbg_index(pp4[h].w, g.n, g.status) : pp4[h].w;
         }
-      } else {
-#pragma unroll
-        for (int d = 0; d < kBufs; ++d)
-#pragma unroll
-          for (int u = 0; u < kRegs; ++u) {
-            const long long t = (g0 + d) * kWinSlots + lane + 32 * u;
-            pp[d][u] = (g0 + d < wc && lane + 32 * u < kWinSlots && t < g.P)
-                           ? dbg_index(g.cpins[t], g.n, g.status)
-                           : 0;
-          }
       }
       wl = (lane <= kGroupWin && g0 + lane <= nwin) ? g.win_edge[g0 + lane] : 0;
     };
-    load_group(wb, pc, pc4, wc_e);
+    load_group(wb, pc4, wc_e);
     long long j = wb;
+    int q = 0;
+    uint32_t pe = 1;  // parity of the stage's last release, once it has one
     bool stop = false;
     for (long long g0 = wb; g0 < wc && !stop; g0 += kGroupWin) {
-      load_group(g0 + kGroupWin, pn, pn4, wn_e);
+      load_group(g0 + kGroupWin, pn4, wn_e);
 #pragma unroll
       for (int d = 0; d < kGroupWin; ++d) {
         j = g0 + d;
@@ -420,11 +475,8 @@ __global__ void __launch_bounds__(kBulkThreads, 1)
           stop = true;
           break;
         }
-        const int q = (int)((j - wb) % nst);
-        const long long use = (j - wb) / nst;
-        if (use > 0) {
-          const bool ok = __all_sync(0xffffffffu, mbar_wait(&empty[q], (uint32_t)((use - 1) & 1),
-                                                            kCopyWaitIters));
+        if (j - wb >= nst) {
+          const bool ok = __all_sync(0xffffffffu, mbar_wait(&empty[q], pe, kCopyWaitIters));
           if (!ok) {
             fail();
             stop = true;
@@ -439,9 +491,9 @@ __global__ void __launch_bounds__(kBulkThreads, 1)
         const int c0 = ef & ~3, cn = ((el + 4) & ~3) - c0;
         const int w0 = ef & ~(kWv - 1), wn = ((el + kWv - 1) & ~(kWv - 1)) - w0;
         const bool mok = el >= ef && el - ef + 8 <= kMetaEdges;
-        const int copied = G4 ? (rows + 3) / 4 * 4 : rows;  // gather4 moves whole groups of four
-        const uint32_t bytes =
-            (uint32_t)copied * row_bytes + (mok ? (uint32_t)(cn * 4 + wn * (int)sizeof(T)) : 0u);
+        const uint32_t bytes =  // gather4 moves whole groups of four rows
+            (uint32_t)((rows + 3) / 4 * 4 * pw * (int)sizeof(T)) +
+            (mok ? (uint32_t)(cn * 4 + wn * (int)sizeof(T)) : 0u);
         if (lane == 0) {
           meta[q][0] = ef;
           meta[q][1] = el;
@@ -449,50 +501,64 @@ __global__ void __launch_bounds__(kBulkThreads, 1)
           mbar_arrive_expect_tx(&full[q], bytes);
         }
         __syncwarp();
-        T* dst = ring + (size_t)q * kWinSlots * pitch;
-        if constexpr (G4) {
-          const int r4 = 4 * (lane & 15);
-          if ((lane >> 4) == (d & 1) && r4 < rows) {
-            const int4 pv = pc4[d >> 1];
-            // rows past the window's end repeat its row r4
-            gather4_g2s(dst + (size_t)r4 * pitch, &tmap, pv.x, r4 + 1 < rows ? pv.y : pv.x,
-                        r4 + 2 < rows ? pv.z : pv.x, r4 + 3 < rows ? pv.w : pv.x, &full[q]);
-          }
-        } else {
-#pragma unroll
-          for (int u = 0; u < kRegs; ++u) {
-            const int r = lane + 32 * u;
-            if (r < rows)
-              bulk_g2s(dst + (size_t)r * pitch, Q + (long long)pc[d][u] * ldq, row_bytes, &full[q]);
-          }
+        T* dst = ring + (size_t)q * kWinSlots * pw;
+        const int r4 = 4 * (lane & 15);
+        if ((lane >> 4) == (d & 1) && r4 < rows) {
+          const int4 pv = pc4[d >> 1];
+          // rows past the window's end repeat its row r4
+          gather4_g2s(dst + (size_t)r4 * pw, &tmap, col0, pv.x, r4 + 1 < rows ? pv.y : pv.x,
+                      r4 + 2 < rows ? pv.z : pv.x, r4 + 3 < rows ? pv.w : pv.x, &full[q]);
         }
         if (mok && lane == 0) {
           bulk_g2s(&m_ceptr[q][0], g.ceptr + c0, (uint32_t)cn * 4u, &full[q]);
           if (wn > 0) bulk_g2s(&m_ew[q][0], ewT + w0, (uint32_t)(wn * sizeof(T)), &full[q]);
         }
         j = j + 1;
+        if (++q == nst) q = 0, pe ^= 1u;
       }
 #pragma unroll
-      for (int d = 0; d < kBufs; ++d) {
-        pc4[d] = pn4[d];
-#pragma unroll
-        for (int u = 0; u < kRegs; ++u) pc[d][u] = pn[d][u];
-      }
+      for (int d = 0; d < kBufs; ++d) pc4[d] = pn4[d];
       wc_e = wn_e;
     }
     if (lane == 0) issued = j;
   } else {
     // ---- consumers
     const int cw = wid - 1;
-    T pacc[NC];
+    const int nchunk = (pcols + V - 1) / V;
+    const int slot_end = (int)min(wc * kWinSlots, (long long)g.P);
+    T pacc[N];
 #pragma unroll
-    for (int c = 0; c < NC; ++c) pacc[c] = 0;
-    for (long long w = wb; w < we; ++w) {
-      const int q = (int)((w - wb) % nst);
-      bool got = mbar_wait(&full[q], (uint32_t)(((w - wb) / nst) & 1), kCopyWaitIters);
-      if (w + 1 < wc)
-        got = got && mbar_wait(&full[(w + 1 - wb) % nst], (uint32_t)(((w + 1 - wb) / nst) & 1),
-                               kCopyWaitIters);
+    for (int q = 0; q < N; ++q) pacc[q] = 0;
+    // the groups' sums of a column meet by halves: group bit o keeps one half
+    // of its values and takes the partner's copy of that half
+    auto flush = [&]() {
+#pragma unroll
+      for (int h = kGrps / 2; h >= 1; h >>= 1) {
+        const bool up = (grp & h) != 0;
+        const int keep = NA * h;
+#pragma unroll
+        for (int q = 0; q < N / 2; ++q) {
+          if (q < keep) {
+            const T send = up ? pacc[q] : pacc[q + keep];
+            const T mine = up ? pacc[q + keep] : pacc[q];
+            pacc[q] = mine + __shfl_xor_sync(0xffffffffu, send, h * kEdgeLanes);
+          }
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < NA; ++q) acc[q] += (double)pacc[q];
+#pragma unroll
+      for (int q = 0; q < N; ++q) pacc[q] = 0;
+    };
+    // window w sits in stage q, the next one in stage qn (parities pq, pn);
+    // kept as counters: a window's share of a warp is a few hyperedges, and
+    // divisions per window cost as much as those
+    int q = 0, qn = nst > 1 ? 1 : 0;
+    uint32_t pn = 0;
+    const int nw = (int)(we - wb), nc = (int)(wc - wb);
+    bool got = nw == 0 || mbar_wait(&full[0], 0u, kCopyWaitIters);
+    for (int w = 0; w < nw; ++w) {
+      if (w + 1 < nc) got = got && mbar_wait(&full[qn], pn, kCopyWaitIters);
       got = __all_sync(0xffffffffu, got);
       if (!got || *abort_v) {
         if (!got) fail();
@@ -502,58 +568,94 @@ __global__ void __launch_bounds__(kBulkThreads, 1)
       const bool mok = meta[q][2] != 0;
       const int c0 = ef & ~3, w0 = ef & ~(16 / (int)sizeof(T) - 1);
       const int row_w = q * kWinSlots;  // ring row of the window's first slot
-      const long long slot_w = w * kWinSlots;
-      const long long slot_end = min(wc * kWinSlots, (long long)g.P);
-      for (int e = ef + cw; e < el; e += kConsumers) {
-        int a, b;
-        T we_;
-        if (mok) a = m_ceptr[q][e - c0], b = m_ceptr[q][e + 1 - c0], we_ = m_ew[q][e - w0];
-        else a = g.ceptr[e], b = g.ceptr[e + 1], we_ = ewT[e];
-        const int k = b - a;
-        // staged: slots [w kWinSlots, min(wc kWinSlots, P)); a >= w kWinSlots
-        if (k < 2 || k > kBigEdge || (long long)b > slot_end) continue;
-        const int r0 = row_w + (int)(a - slot_w);  // ring row of the first pin
-        T mx[NC], mn[NC];
+      const int slot_w = (int)((wb + w) * kWinSlots);
+      const int q0 = ef / kGrps;  // first quad; this warp's are cw mod kConsumers
+      for (int qd = q0 + (cw + kConsumers - q0 % kConsumers) % kConsumers; qd * kGrps < el; qd += kConsumers) {
+        const int e = qd * kGrps + grp;
+        int a = 0, k = 0;
+        T we_ = 0;
+        if (e >= ef && e < el) {
+          int b;
+          if (mok) a = m_ceptr[q][e - c0], b = m_ceptr[q][e + 1 - c0], we_ = m_ew[q][e - w0];
+          else a = g.ceptr[e], b = g.ceptr[e + 1], we_ = ewT[e];
+          k = b - a;
+          // staged: slots [w kWinSlots, min(wc kWinSlots, P)); a >= w kWinSlots
+          if (k < 2 || k > kBigEdge || b > slot_end) k = 0;
+        }
+        const int r0 = row_w + (a - slot_w);  // ring row of the first pin
+        Extrema<T> ex[C][V];
+        // first round: each group its own hyperedge of up to kGroupPins pins;
+        // then hyperedges with more, one at a time, all groups sharing the
+        // pins (a window's stage is held until its longest hyperedge is done)
+        unsigned todo = __ballot_sync(0xffffffffu, sub == 0 && k > kGroupPins);
+        int src = -1;
+        while (true) {
+          const int rr = src < 0 ? r0 : __shfl_sync(0xffffffffu, r0, src);
+          const int kk = src < 0 ? (k <= kGroupPins ? k : 0) : __shfl_sync(0xffffffffu, k, src);
+          const int step = src < 0 ? 1 : kGrps;
 #pragma unroll
-        for (int c = 0; c < NC; ++c) mx[c] = lowest<T>(), mn[c] = -lowest<T>();
-        for (int t = 0; t < k; t += 4) {
-          const T* rp[4];
+          for (int c = 0; c < C; ++c)
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            int x = r0 + min(t + u, k - 1);
-            x = x >= ring_rows ? x - ring_rows : x;
-            rp[u] = ring + x * pitch + lane;
-          }
+            for (int v = 0; v < V; ++v) ex[c][v].clear();
+          for (int t = src < 0 ? 0 : grp; t < kk; t += 2 * step) {
+            int x0 = rr + t, x1 = rr + (t + step < kk ? t + step : t);
+            x0 = x0 >= ring_rows ? x0 - ring_rows : x0;
+            x1 = x1 >= ring_rows ? x1 - ring_rows : x1;
+            const uint4* p0 = reinterpret_cast<const uint4*>(ring + x0 * pw) + sub;
+            const uint4* p1 = reinterpret_cast<const uint4*>(ring + x1 * pw) + sub;
 #pragma unroll
-          for (int c = 0; c < NC; ++c) {
-            if (lane + 32 * c < K) {
-              const T v0 = rp[0][32 * c], v1 = rp[1][32 * c];
-              const T v2 = rp[2][32 * c], v3 = rp[3][32 * c];
-              mx[c] = fmax(fmax(mx[c], fmax(v0, v1)), fmax(v2, v3));
-              mn[c] = fmin(fmin(mn[c], fmin(v0, v1)), fmin(v2, v3));
+            for (int c = 0; c < C; ++c) {
+              if (sub + kEdgeLanes * c < nchunk) {
+                T v0[V], v1[V];
+                const uint4 u0 = p0[kEdgeLanes * c], u1 = p1[kEdgeLanes * c];
+                memcpy(v0, &u0, 16);
+                memcpy(v1, &u1, 16);
+#pragma unroll
+                for (int v = 0; v < V; ++v) ex[c][v].add(v0[v]), ex[c][v].add(v1[v]);
+              }
             }
           }
-        }
+          if (src >= 0) {
 #pragma unroll
-        for (int c = 0; c < NC; ++c) {
-          const int col = lane + 32 * c;
-          const T sp = mx[c] - mn[c];
-          if (col < K) {
-            pacc[c] += we_ * sp * sp;
-            if (spread) spread[(long long)e * ldsp + col] = sp;
+            for (int c = 0; c < C; ++c)
+#pragma unroll
+              for (int v = 0; v < V; ++v)
+#pragma unroll
+                for (int o = kEdgeLanes; o < 32; o <<= 1) ex[c][v].join(o);
           }
-        }
-      }
-      // partial sums in the working type over kFlushWin windows; FP64 beyond
-      if ((w - wb) % kFlushWin == kFlushWin - 1) {
+          if (kk > 0 && (src < 0 || grp == src / kEdgeLanes)) {
+            uint4* row = reinterpret_cast<uint4*>(spread + (long long)e * ldsp + col0) + sub;
 #pragma unroll
-        for (int c = 0; c < NC; ++c) acc[c] += (double)pacc[c], pacc[c] = 0;
+            for (int c = 0; c < C; ++c) {
+              if (sub + kEdgeLanes * c < nchunk) {
+                T sp[V];
+#pragma unroll
+                for (int v = 0; v < V; ++v) {
+                  sp[v] = ex[c][v].spread();
+                  pacc[c * V + v] += we_ * sp[v] * sp[v];
+                }
+                if (spread) {  // rows are padded to 16 bytes
+                  uint4 u;
+                  memcpy(&u, sp, 16);
+                  row[kEdgeLanes * c] = u;
+                }
+              }
+            }
+          }
+          if (!todo) break;
+          src = __ffs(todo) - 1;
+          todo &= todo - 1;
+        }
       }
       __syncwarp();
+      // partial sums in the working type over kFlushWin windows; FP64 beyond
+      if (w % kFlushWin == kFlushWin - 1) flush();
       if (lane == 0) mbar_arrive(&empty[q]);
+      q = qn;
+      if (++qn == nst) qn = 0, pn ^= 1u;
     }
-#pragma unroll
-    for (int c = 0; c < NC; ++c) acc[c] += (double)pacc[c];
+    __syncwarp();
+    flush();
   }
   __syncthreads();
   // every copy has landed before the ring is reused or the CTA exits: the
@@ -562,17 +664,32 @@ __global__ void __launch_bounds__(kBulkThreads, 1)
     for (long long j = issued - nst > wb ? issued - nst : wb; j < issued; ++j)
       mbar_wait(&full[(j - wb) % nst], (uint32_t)(((j - wb) / nst) & 1), kCopyWaitIters);
   __syncthreads();
-  // per-warp sums in the (now idle) ring: [warp][32 NC]
+  // per-warp sums in the (now idle) ring: [warp][kPartChunks kEdgeLanes V]
+  constexpr int kCols = kPartChunks * kEdgeLanes * V;
   double* wred = reinterpret_cast<double*>(ring_raw);
+  if (wid > 0) {
+    // value q of the flush's order: the halves kept at each level, from the top
+    int first = 0;
 #pragma unroll
-  for (int c = 0; c < NC; ++c) wred[wid * 32 * NC + lane + 32 * c] = acc[c];
+    for (int h = kGrps / 2; h >= 1; h >>= 1) first += (grp & h) ? NA * h : 0;
+#pragma unroll
+    for (int q = 0; q < NA; ++q) {
+      const int idx = first + q;
+      if (idx < C * V) wred[(wid - 1) * kCols + (sub + kEdgeLanes * (idx / V)) * V + idx % V] = acc[q];
+    }
+  }
   __syncthreads();
+  // k_score_big1 (bpart) complete: a no-op unless this pass was launched as
+  // its programmatic dependent
+  pdl_wait();
   for (int col = threadIdx.x; col < K; col += blockDim.x) {
-    double sum = 0.0;
-    for (int w = 0; w < kBulkThreads / 32; ++w) sum += wred[w * 32 * NC + col];
+    double sum = big_share(bpart, nbpart, K, col);
+    const int c = col - col0;
+    if (c >= 0 && c < pcols)
+      for (int w = 0; w < kConsumers; ++w) sum += wred[w * kCols + c];
     red.part[(size_t)blockIdx.x * K + col] = sum;
   }
-  finish_qh<NC>(red, K, bpart, nbpart, QH, invQH, QH_out);
+  finish_qh<16>(red, K, QH, invQH, QH_out);
 }
 
 // Pass 2 for one hyperedge whose extrema a warp holds (lanes over columns):
@@ -1072,51 +1189,56 @@ hef_status launch_score(const hef_incidence* inc, const T* Q, long long ldq, int
   const int ldsp = spread_ld(K, sizeof(T));
   HEF_LAUNCH("k_score_big1", st, k_score_big1<T, NC><<<w.bgrid, kThreads, 0, st>>>(g, Q, ldq, K, w.bpart,
                                                                                    spread, ldsp));
-  // pass 1 staged through shared memory when the rows can be bulk-copied
-  // (16-byte aligned rows; a row pitch of 16-byte multiples) and at least two
-  // stages fit; by four-row tensor-map gathers when a box row (K rounded up
-  // to 32 bytes, at most 256 elements) fits in the pitch; otherwise the warps
-  // gather the rows
+  // pass 1 staged through shared memory when a tensor map can address the rows
+  // (16-byte aligned rows, a pitch of 16-byte multiples); otherwise the warps
+  // gather the rows.  Parts of at most kPartChunks chunks per lane (768 bytes),
+  // as equal as the 32-byte rounding allows
   const bool aligned = (reinterpret_cast<uintptr_t>(Q) % 16 == 0) && ((size_t)ldq * sizeof(T)) % 16 == 0;
-  const int bw = (int)(((size_t)K * sizeof(T) + 31) / 32 * 32 / sizeof(T));
+  constexpr int kRound = 32 / (int)sizeof(T);
+  constexpr int kMaxPart = kPartChunks * kEdgeLanes * 16 / (int)sizeof(T);
+  const int want = (K + kMaxPart - 1) / kMaxPart;
+  const int pw = ((K + want - 1) / want + kRound - 1) / kRound * kRound;
+  const int parts = (K + pw - 1) / pw;
   CUtensorMap tmap;
   memset(&tmap, 0, sizeof(tmap));
-  bool g4 = aligned && bw <= 256 && bw <= ldq && encode_rows_map(&tmap, Q, ldq, inc->n, bw);
-  const uint32_t row_bytes = g4 ? (uint32_t)(bw * sizeof(T)) : (uint32_t)(((size_t)K * sizeof(T) + 15) / 16 * 16);
-  const size_t stage_bytes = (size_t)kWinSlots * row_bytes;
+  const size_t stage_bytes = (size_t)kWinSlots * pw * sizeof(T);
   // stages: as many as fit next to the kernel's static shared memory (and
   // 128 bytes to align the ring)
-  static thread_local int stat = -1;  // static bytes of this instantiation
+  static thread_local int stat = -1;  // largest static bytes over the instantiations
   if (stat < 0) {
     cudaFuncAttributes fa;
-    HEF_CHECK_CUDA(cudaFuncGetAttributes(&fa, k_score_pass1_bulk<T, NC, true>));
+    HEF_CHECK_CUDA(cudaFuncGetAttributes(&fa, k_score_pass1_bulk<T, kPartChunks>));
     stat = (int)fa.sharedSizeBytes;
   }
   const size_t avail = kStageSmem > (size_t)stat + 128 ? kStageSmem - stat - 128 : 0;
   const int nst = (int)std::min<size_t>(kMaxStages, avail / stage_bytes);
   // the ring also holds the per-warp sums at the end
   const size_t smem =
-      std::max(nst * stage_bytes, (size_t)(kBulkThreads / 32) * 32 * NC * sizeof(double)) + 128;
-  const bool bulk = aligned && nst >= 2 && smem + stat <= kMaxSmemOptin && num_sms() <= w.grid;
+      std::max(nst * stage_bytes, (size_t)kConsumers * kMaxPart * sizeof(double)) + 128;
+  const bool bulk = aligned && nst >= 2 && smem + stat <= kMaxSmemOptin && num_sms() <= w.grid &&
+                    parts <= num_sms() && encode_rows_map(&tmap, Q, ldq, inc->n, pw);
   if (bulk) {
-    const int pitch = (int)(row_bytes / sizeof(T));
-    if (g4) {
-      HEF_ENSURE_SMEM((k_score_pass1_bulk<T, NC, true>), (int)smem);
+    auto launch = [&](auto kernel) -> hef_status {
+      HEF_ENSURE_SMEM(kernel, (int)smem);
       // a programmatic dependent of k_score_big1: it runs beside it and waits
       // for it only before the reduction that reads bpart
       HEF_LAUNCH("k_score_pass1", st,
                  HEF_CHECK_CUDA(launch_dependent_smem(
-                     k_score_pass1_bulk<T, NC, true>, num_sms(), kBulkThreads, smem, st, g, Q, ldq, K,
-                     pitch, row_bytes, nst, red, w.bpart, w.bgrid, w.QH, w.invQH, QH_out, spread, ldsp,
-                     scal_view<T>(inc).ew, inc->status, tmap)));
-    } else {
-      HEF_ENSURE_SMEM((k_score_pass1_bulk<T, NC, false>), (int)smem);
-      HEF_LAUNCH("k_score_pass1", st,
-                 HEF_CHECK_CUDA(launch_dependent_smem(
-                     k_score_pass1_bulk<T, NC, false>, num_sms(), kBulkThreads, smem, st, g, Q, ldq,
-                     K, pitch, row_bytes, nst, red, w.bpart, w.bgrid, w.QH, w.invQH, QH_out, spread,
-                     ldsp, scal_view<T>(inc).ew, inc->status, tmap)));
+                     kernel, num_sms(), kBulkThreads, smem, st, g, K, parts, pw, nst, red, w.bpart,
+                     w.bgrid, w.QH, w.invQH, QH_out, spread, ldsp, scal_view<T>(inc).ew, inc->status,
+                     tmap)));
+      return HEF_OK;
+    };
+    hef_status s1;
+    switch ((pw + kEdgeLanes * kRound / 2 - 1) / (kEdgeLanes * kRound / 2)) {  // chunks per lane
+      case 1: s1 = launch(k_score_pass1_bulk<T, 1>); break;
+      case 2: s1 = launch(k_score_pass1_bulk<T, 2>); break;
+      case 3: s1 = launch(k_score_pass1_bulk<T, 3>); break;
+      case 4: s1 = launch(k_score_pass1_bulk<T, 4>); break;
+      case 5: s1 = launch(k_score_pass1_bulk<T, 5>); break;
+      default: s1 = launch(k_score_pass1_bulk<T, kPartChunks>); break;
     }
+    if (s1) return s1;
   } else {
     const int g1 = std::min(w.grid, num_sms() * resident_ctas(k_score_pass1<T, NC>, kThreads));
     HEF_LAUNCH("k_score_pass1", st, k_score_pass1<T, NC><<<g1, kThreads, 0, st>>>(
