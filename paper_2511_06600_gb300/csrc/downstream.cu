@@ -232,24 +232,60 @@ __global__ void k_clusters(int n, const int32_t* __restrict__ owner, const int32
   }
 }
 
-template <typename T>
-__device__ __forceinline__ double qval(const T* Q, long long ldq, long long row, int i) {
-  if constexpr (std::is_same<T, __nv_bfloat16>::value) return (double)__bfloat162float(Q[row * ldq + i]);
-  else return (double)Q[row * ldq + i];
+// (double)x by integer operations for normal x: conversions to FP64 share the
+// FP64 pipe's rate of two per clock and SM.
+__device__ __forceinline__ double widen(float x) {
+  const unsigned b = __float_as_uint(x), e = (b >> 23) & 0xffu;
+  if (e - 1u >= 254u) return (double)x;  // zero, subnormal, infinite, NaN
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
 }
 
-// Centroid rows of the contracted supernodes: one warp per supernode, lanes
-// over columns, members summed in the forming hyperedge's pin order.  Also
-// the FP32 rows mu32 and the column scales that k_seeds bounds distances
-// with: scale[i] = 1/Q_H[i] (0 for columns that take no part), scale[K] = 1
-// when some Q_H lies outside [1e-30, 1e30], where FP32 bounds could overflow
-// or underflow and every distance is formed in FP64.
 template <typename T>
-__global__ void k_centroids(int nc, const int32_t* __restrict__ formed_by,
-                            const int* __restrict__ mrow, const int64_t* __restrict__ eptr,
-                            const int32_t* __restrict__ pins, const T* __restrict__ Q, long long ldq,
-                            int K, const double* __restrict__ QH, double* __restrict__ mu,
-                            float* __restrict__ mu32, float* __restrict__ scale) {
+__device__ __forceinline__ double qval(const T* Q, long long ldq, long long row, int i) {
+  if constexpr (std::is_same<T, __nv_bfloat16>::value) return widen(__bfloat162float(Q[row * ldq + i]));
+  else if constexpr (std::is_same<T, float>::value) return widen(Q[row * ldq + i]);
+  else return Q[row * ldq + i];
+}
+
+// a / k rounded to nearest (as __ddiv_rn) for an integer 2 <= k < 2^31 given
+// with rk = 1/k rounded to nearest: q0 is within two ulps, its residual is
+// exact, and the corrected quotient is off by less than 2^-104 of itself before
+// its rounding, while a quotient by k that is no rounding boundary lies at
+// least 2^-54 / k away from one.  Three FP64 operations (one when k is a power
+// of two) instead of a division's eight and its special cases; tiny and
+// non-finite values take the division.
+__device__ __forceinline__ double div_by_int(double a, double k, double rk, bool pow2) {
+  const int f = (__double2hiint(a) >> 20) & 0x7ff;
+  if (f < 200 || f > 2000) return __ddiv_rn(a, k);
+  const double q0 = __dmul_rn(a, rk);
+  if (pow2) return q0;
+  return __fma_rn(__fma_rn(-k, q0, a), rk, q0);
+}
+
+// x truncated to FP32 (rounded where its exponent is out of the normal range).
+__device__ __forceinline__ float narrow(double x) {
+  const unsigned h = (unsigned)__double2hiint(x), f = (h >> 20) & 0x7ffu;
+  if (f < 897u || f > 1150u) return (float)x;
+  return __uint_as_float((h & 0x80000000u) | ((((h & 0x7fffffffu) - (896u << 20)) << 3) |
+                                              ((unsigned)__double2loint(x) >> 29)));
+}
+
+// Centroid rows of the contracted supernodes: one warp per supernode, NC
+// columns per lane, members summed in the forming hyperedge's pin order (one
+// round of row loads per member).  Also what k_seeds reads: the FP32 rows mu32;
+// the column scales scale[i] = 1/Q_H[i] (0 for columns that take no part),
+// scale[K] = 1 when some Q_H lies outside [1e-30, 1e30], where FP32 bounds could
+// overflow or underflow and every distance is formed in FP64; and for every
+// vertex its supernode and that supernode's row, or -1 when it is isolated.
+// Bound by the FP64 pipe (one add per member and column, then the division):
+// 186 -> 152 us at 210,000 vertices, K = 160.
+template <typename T, int NC>
+__global__ void __launch_bounds__(kThreads)
+    k_centroids(int n, const int32_t* __restrict__ formed_by, const int* __restrict__ mrow,
+                const int32_t* __restrict__ cluster, const int64_t* __restrict__ eptr,
+                const int32_t* __restrict__ pins, const T* __restrict__ Q, long long ldq, int K,
+                const double* __restrict__ QH, double* __restrict__ mu, float* __restrict__ mu32,
+                float* __restrict__ scale, int2* __restrict__ vinfo) {
   if (blockIdx.x == 0) {
     int wide = 0;
     for (int i = threadIdx.x; i < K; i += blockDim.x) {
@@ -261,21 +297,40 @@ __global__ void k_centroids(int nc, const int32_t* __restrict__ formed_by,
     wide = __syncthreads_or(wide);
     if (threadIdx.x == 0) scale[K] = wide ? 1.0f : 0.0f;
   }
+  const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (tid < n) {
+    const int cv = cluster[tid];
+    vinfo[tid] = formed_by[cv] >= 0 ? make_int2(cv, mrow[cv]) : make_int2(-1, 0);
+  }
   const int lane = threadIdx.x & 31;
-  const int c = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  if (c >= nc) return;
+  const int c = (int)(tid >> 5);
+  if (c >= n) return;
   const int e = formed_by[c];
   if (e < 0) return;
   const int64_t a = eptr[e], b = eptr[e + 1];
-  const double k = (double)(b - a);
-  double* row = mu + (size_t)mrow[c] * K;
-  float* row32 = mu32 + (size_t)mrow[c] * K;
-  for (int i = lane; i < K; i += 32) {
-    double acc = 0.0;
-    for (int64_t t = a; t < b; ++t) acc = __dadd_rn(acc, qval(Q, ldq, pins[t], i));
-    const double x = __ddiv_rn(acc, k);
-    row[i] = x;
-    row32[i] = (float)x;
+  const double k = (double)(b - a), rk = __ddiv_rn(1.0, k);
+  const bool pow2 = ((b - a) & (b - a - 1)) == 0;
+  double acc[NC];
+#pragma unroll
+  for (int j = 0; j < NC; ++j) acc[j] = 0.0;
+  for (int64_t t = a; t < b; ++t) {
+    const int u = pins[t];
+    double x[NC];
+#pragma unroll
+    for (int j = 0; j < NC; ++j) x[j] = lane + 32 * j < K ? qval(Q, ldq, u, lane + 32 * j) : 0.0;
+#pragma unroll
+    for (int j = 0; j < NC; ++j)
+      if (32 * j < K) acc[j] = __dadd_rn(acc[j], x[j]);  // no FP64 for absent columns
+  }
+  const size_t row = (size_t)mrow[c] * K;
+#pragma unroll
+  for (int j = 0; j < NC; ++j) {
+    const int i = lane + 32 * j;
+    if (i < K) {
+      const double x = div_by_int(acc[j], k, rk, pow2);
+      mu[row + i] = x;
+      mu32[row + i] = narrow(x);
+    }
   }
 }
 
@@ -286,27 +341,33 @@ __global__ void k_centroids(int nc, const int32_t* __restrict__ formed_by,
 //
 // The scores are FP64 (round to nearest), and FP64 division is what bound this
 // kernel (two DFMA per clock and SM): K divisions per candidate pin, 5.68 ms at
-// 210,000 vertices, K = 160; 0.95 ms now.  A candidate is now bounded in FP32 first: with
-// q, m the FP32 roundings of Q[p,i] and mu_c[i], |Q - mu| lies within
-// err = 2^-23 (|q| + |m|) of |q - m|, which gives [lb_i, ub_i] around each
+// 210,000 vertices, K = 160; 0.46 ms now.  A candidate is now bounded in FP32 first: with
+// q, m the FP32 values of Q[p,i] and mu_c[i] (rounded and truncated), |Q - mu|
+// lies within err = 1.5 2^-23 (|q| + |m|) of |q - m|, which gives [lb_i, ub_i] around each
 // column's ratio and [max lb, max ub] around the score (the constants below
 // leave slack for every rounding, underflow included).  A candidate whose lower
 // bound exceeds an earlier candidate's upper bound cannot win; for the others
 // only the columns with ub_i >= max lb can hold the maximum, and only those
 // are formed in FP64: one or two divisions for a few candidates per vertex,
 // with the same result bit for bit.  Columns are held NC per lane, so a
-// candidate costs one FP32 row of gathers.
+// candidate costs one FP32 row of gathers.  What remained was the chain of
+// dependent loads from a vertex to its candidates' rows, walked once per
+// hyperedge: the lanes now take the pins of up to 32 hyperedges together, 32
+// pins at a time, which walks it once for most vertices.
+// CTAs of two warps: a CTA keeps its registers until its slowest vertex is done,
+// and about half the vertices have nothing to do.
+constexpr int kSeedThreads = 64;
+
 template <typename T, int NC>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kSeedThreads)
     k_seeds(int n, const int32_t* __restrict__ owner, const int32_t* __restrict__ vptr,
             const int32_t* __restrict__ vedge, const int32_t* __restrict__ perm,
             const int64_t* __restrict__ eptr, const int32_t* __restrict__ pins,
-            const int32_t* __restrict__ cluster, const int32_t* __restrict__ formed_by,
-            const int* __restrict__ mrow, const double* __restrict__ mu,
+            const int2* __restrict__ vinfo, const double* __restrict__ mu,
             const float* __restrict__ mu32, const float* __restrict__ scale,
             const T* __restrict__ Q, long long ldq, int K, const double* __restrict__ QH,
             int32_t* __restrict__ target, double* __restrict__ dist) {
-  constexpr float kErr = 1.3e-7f;       // > 2^-23
+  constexpr float kErr = 1.9e-7f;       // > 1.5 2^-23
   constexpr float kSlack = 1e-6f;       // relative, > the products' and scales' roundings
   constexpr float kTiny = 1e-37f;       // absolute, > what underflow loses
   const int lane = threadIdx.x & 31;
@@ -327,51 +388,89 @@ __global__ void __launch_bounds__(kThreads)
   int best = -1;
   double bd = INFINITY;
   float bound = INFINITY;  // smallest upper bound of a candidate so far
-  for (int t = vptr[p]; t < vptr[p + 1]; ++t) {
-    const int e = perm[vedge[t]];
-    const int64_t b = eptr[e + 1];
-    for (int64_t s0 = eptr[e]; s0 < b; s0 += 32) {
+  const int t1 = vptr[p + 1];
+  for (int t0 = vptr[p]; t0 < t1; t0 += 32) {
+    // lane l: the pins [first, first + cnt) of hyperedge t0 + l, at [at, at +
+    // cnt) of the round's pins
+    int64_t first = 0;
+    int cnt = 0;
+    if (t0 + lane < t1) {
+      const int e = perm[vedge[t0 + lane]];
+      first = eptr[e];
+      cnt = (int)(eptr[e + 1] - first);
+    }
+    int end = cnt;  // inclusive sum over the lanes
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, end, o);
+      if (lane >= o) end += x;
+    }
+    const int total = __shfl_sync(0xffffffffu, end, 31);
+    const int at = end - cnt;
+    for (int s0 = 0; s0 < total; s0 += 32) {
+      // pin s0 + lane lies in the hyperedge of the last lane whose start is at
+      // or before it (empty hyperedges share their successor's start)
+      int h = 0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+        if (__shfl_sync(0xffffffffu, at, h + o) <= s0 + lane) h += o;
+      const int64_t hf = __shfl_sync(0xffffffffu, (long long)first, h);
+      const int ha = __shfl_sync(0xffffffffu, at, h);
       int c = -1 - lane, row = 0;
-      if (s0 + lane < b) {
-        const int u = pins[s0 + lane];
-        const int cu = cluster[u];
-        if (u != p && formed_by[cu] >= 0) c = cu, row = mrow[cu];
+      if (s0 + lane < total) {
+        const int u = pins[hf + (s0 + lane - ha)];
+        const int2 v = vinfo[u];
+        if (u != p && v.x >= 0) c = v.x, row = v.y;
       }
       // each supernode once per 32 pins
       const unsigned peers = __match_any_sync(0xffffffffu, c);
       unsigned todo = __ballot_sync(0xffffffffu, c >= 0 && lane == __ffs(peers) - 1);
+      // bounds of every candidate first, kept by its lane; then FP64 for those
+      // that the smallest upper bound leaves (a warp's FP64 operation takes 16
+      // cycles of the SM's pipe however few of its lanes are on)
+      auto bounds = [&](size_t ro, float (&ub)[NC], float& lo, float& hi) {
+        float m[NC];
+#pragma unroll
+        for (int j = 0; j < NC; ++j) m[j] = lane + 32 * j < K ? mu32[ro + lane + 32 * j] : 0.0f;
+        lo = 0.0f, hi = 0.0f;
+        bool open = false;  // overflow or NaN: no upper bound
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+          if (32 * j < K) {
+            const float d = fabsf(q[j] - m[j]), size = fabsf(q[j]) + fabsf(m[j]);
+            const float du = fmaf(kErr, size, d), dl = fmaxf(fmaf(-kErr, size, d), 0.0f);
+            ub[j] = du * sc[j] * du;
+            open |= !(ub[j] <= 3.0e38f);
+            hi = fmaxf(hi, ub[j]);
+            lo = fmaxf(lo, dl * sc[j] * dl);
+          }
+        }
+        // non-negative floats order as their bits
+        hi = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(open ? INFINITY : hi)));
+        lo = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(lo)));
+        hi = hi * (1.0f + kSlack) + kTiny;
+        lo = fmaxf(fminf(lo, 3.0e38f) * (1.0f - kSlack) - kTiny, 0.0f);
+        if (wide) lo = 0.0f, hi = INFINITY;
+      };
+      float ub[NC], lo, hi, mylo = INFINITY;
+      for (unsigned rest = todo; rest; rest &= rest - 1) {
+        const int src = __ffs(rest) - 1;
+        bounds((size_t)__shfl_sync(0xffffffffu, row, src) * K, ub, lo, hi);
+        if (lane == src) mylo = lo;
+        bound = fminf(bound, hi);
+      }
+      todo = __ballot_sync(0xffffffffu, ((todo >> lane) & 1u) && mylo <= bound);
       while (todo) {
         const int src = __ffs(todo) - 1;
         todo &= todo - 1;
         const int cc = __shfl_sync(0xffffffffu, c, src);
         const size_t ro = (size_t)__shfl_sync(0xffffffffu, row, src) * K;
-        float m[NC], ub[NC];
-#pragma unroll
-        for (int j = 0; j < NC; ++j) m[j] = lane + 32 * j < K ? mu32[ro + lane + 32 * j] : 0.0f;
-        float lo = 0.0f, hi = 0.0f;
-#pragma unroll
-        for (int j = 0; j < NC; ++j) {
-          const float d = fabsf(q[j] - m[j]);
-          const float err = kErr * (fabsf(q[j]) + fabsf(m[j]));
-          const float du = d + err, dl = d - err;
-          float u = du * sc[j] * du;
-          u = u * (1.0f + kSlack) + kTiny;
-          if (!(u <= 3.0e38f)) u = INFINITY;  // overflow or NaN: no bound
-          ub[j] = u;
-          hi = fmaxf(hi, u);
-          if (dl > 0.0f) lo = fmaxf(lo, fminf(dl * sc[j] * dl * (1.0f - kSlack), 3.0e38f) - kTiny);
-        }
-        // non-negative floats order as their bits
-        hi = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(hi)));
-        lo = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(lo)));
-        if (wide) lo = 0.0f, hi = INFINITY;
-        if (lo > bound) continue;
-        bound = fminf(bound, hi);
+        bounds(ro, ub, lo, hi);
         double d = 0.0;
 #pragma unroll
         for (int j = 0; j < NC; ++j) {
           const int i = lane + 32 * j;
-          if (i < K && (wide || !(ub[j] < lo))) {
+          if (i < K && (wide || !(ub[j] * (1.0f + kSlack) + kTiny < lo))) {
             const double qh = QH[i];
             if (qh > 1e-300) {
               const double diff = __dsub_rn(qval(Q, ldq, p, i), mu[ro + i]);
@@ -380,11 +479,10 @@ __global__ void __launch_bounds__(kThreads)
             }
           }
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const double x = __shfl_xor_sync(0xffffffffu, d, o);
-          d = x > d ? x : d;
-        }
+        // the largest of the lanes' non-negative doubles, by their bits
+        const unsigned dh = (unsigned)__double2hiint(d), mh = __reduce_max_sync(0xffffffffu, dh);
+        const unsigned ml = __reduce_max_sync(0xffffffffu, dh == mh ? (unsigned)__double2loint(d) : 0u);
+        d = __hiloint2double((int)mh, (int)ml);
         if (d < bd || (d == bd && cc < best)) best = cc, bd = d;
       }
     }
@@ -622,6 +720,7 @@ struct LevelWs {
   double* eta_next;
   double* eta2;
   double* mu;
+  int2* vinfo;   // n: supernode and its centroid row, or -1
   float* mu32;   // FP32 rows of mu, scale (K + 1): bounds of the seeds' distances
   float* scale;
   int* minv;
@@ -655,6 +754,7 @@ size_t carve_level(void* base, long long n, long long m, int K, LevelWs* w) {
   w->mu = c.take<double>((size_t)(n / 2 + 1) * (K > 0 ? K : 1));
   w->mu32 = c.take<float>((size_t)(n / 2 + 1) * (K > 0 ? K : 1));
   w->scale = c.take<float>(K + 1);
+  w->vinfo = c.take<int2>(K > 0 ? n + 1 : 1);
   w->minv = c.take<int>(n + 1);
   w->keep = c.take<int>(m + 1);
   w->ne = c.take<int>(m + 1);
@@ -810,22 +910,22 @@ extern "C" hef_status hef_coarsen_level(const hef_incidence* inc, const int64_t*
     const int wgrid = (int)((n * 32 + kThreads - 1) / kThreads);
     auto run = [&](auto tag) -> hef_status {
       using QT = decltype(tag);
-      HEF_LAUNCH("k_centroids", st, k_centroids<QT><<<wgrid, kThreads, 0, st>>>(
-                                        nn, ws.formed_by, ws.cflag, eptr, pins,
-                                        static_cast<const QT*>(Q), ldq, K, QH, ws.mu, ws.mu32,
-                                        ws.scale));
-      auto seeds = [&](auto kernel) {
-        HEF_LAUNCH("k_seeds", st, kernel<<<wgrid, kThreads, 0, st>>>(
-                                      nn, out->owner, g.vptr, g.vedge, g.perm, eptr, pins,
-                                      out->cluster, ws.formed_by, ws.cflag, ws.mu, ws.mu32,
-                                      ws.scale, static_cast<const QT*>(Q), ldq, K, QH,
-                                      out->target, out->dist));
-      };
       // columns per lane: enough registers for K, no more than it needs
-      if (K <= 64) seeds(k_seeds<QT, 2>);
-      else if (K <= 128) seeds(k_seeds<QT, 4>);
-      else if (K <= 256) seeds(k_seeds<QT, 8>);
-      else seeds(k_seeds<QT, 16>);
+      auto cluster_seeds = [&](auto centroids, auto seeds) {
+        HEF_LAUNCH("k_centroids", st, centroids<<<wgrid, kThreads, 0, st>>>(
+                                          nn, ws.formed_by, ws.cflag, out->cluster, eptr, pins,
+                                          static_cast<const QT*>(Q), ldq, K, QH, ws.mu, ws.mu32,
+                                          ws.scale, ws.vinfo));
+        HEF_LAUNCH("k_seeds", st, seeds<<<(int)((n * 32 + kSeedThreads - 1) / kSeedThreads), kSeedThreads, 0, st>>>(
+                                      nn, out->owner, g.vptr, g.vedge, g.perm, eptr, pins, ws.vinfo,
+                                      ws.mu, ws.mu32, ws.scale, static_cast<const QT*>(Q), ldq, K,
+                                      QH, out->target, out->dist));
+      };
+      if (K <= 64) cluster_seeds(k_centroids<QT, 2>, k_seeds<QT, 2>);
+      else if (K <= 128) cluster_seeds(k_centroids<QT, 4>, k_seeds<QT, 4>);
+      else if (K <= 192) cluster_seeds(k_centroids<QT, 6>, k_seeds<QT, 6>);
+      else if (K <= 256) cluster_seeds(k_centroids<QT, 8>, k_seeds<QT, 8>);
+      else cluster_seeds(k_centroids<QT, 16>, k_seeds<QT, 16>);
       return HEF_OK;
     };
     if (dtype == HEF_F64) HEF_PASS(run(double{}));
