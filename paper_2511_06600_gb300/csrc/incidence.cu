@@ -58,7 +58,10 @@ __device__ __forceinline__ int block_exclusive_scan_1024(int v, int* total) {
   return incl - v;
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan1(const int* in, int* out, int N, int ntiles,
+// in(i) gives item i; out(i, sum, item) takes its exclusive sum and out(N,
+// total, 0) the total.
+template <typename In, typename Out>
+__global__ void __launch_bounds__(kScanThreads) k_scan1(In in, Out out, int N, int ntiles,
                                                         unsigned int* tctr,
                                                         unsigned long long* stat,
                                                         unsigned int* err) {
@@ -71,7 +74,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan1(const int* in, int* out,
   int sum = 0;
 #pragma unroll
   for (int j = 0; j < kItems; ++j) {
-    v[j] = base + j < N ? in[base + j] : 0;
+    v[j] = base + j < N ? in(base + j) : 0;
     sum += v[j];
   }
   int total;
@@ -116,10 +119,60 @@ __global__ void __launch_bounds__(kScanThreads) k_scan1(const int* in, int* out,
   int run = s_excl + local;
 #pragma unroll
   for (int j = 0; j < kItems; ++j) {
-    if (base + j < N) out[base + j] = run;
+    if (base + j < N) out(base + j, run, v[j]);
     run += v[j];
   }
-  if (t == ntiles - 1 && threadIdx.x == 0) out[N] = s_excl + total;
+  if (t == ntiles - 1 && threadIdx.x == 0) out(N, s_excl + total, 0);
+}
+
+struct ScanIn {
+  const int* in;
+  __device__ int operator()(long long i) const { return in[i]; }
+};
+struct ScanOut {
+  int* out;
+  __device__ void operator()(long long i, int sum, int) const { out[i] = sum; }
+};
+// Pin counts of the hyperedges in the order of the locality schedule (none
+// when the input was rejected, whose offsets mean nothing).
+struct SizesIn {
+  const int64_t* eptr;
+  const int32_t* sched;
+  const unsigned int* status;
+  __device__ int operator()(long long i) const {
+    if (status[0]) return 0;
+    const int e = sched[i];
+    return (int)(eptr[e + 1] - eptr[e]);
+  }
+};
+// Hyperedges with more than kBigEdge pins (internal order): positions in the
+// list, and the list itself.
+struct BigIn {
+  const int32_t* ceptr;
+  const unsigned int* status;
+  __device__ int operator()(long long i) const {
+    return !status[0] && ceptr[i + 1] - ceptr[i] > kBigEdge ? 1 : 0;
+  }
+};
+struct BigOut {
+  int32_t* pos;
+  int32_t* idx;
+  __device__ void operator()(long long i, int sum, int item) const {
+    pos[i] = sum;
+    if (item) idx[sum] = (int32_t)i;
+  }
+};
+
+// One scan of N > 0 items over a zeroed state (bsum: see exclusive_scan).
+template <typename In, typename Out>
+hef_status scan_with(In in, Out out, long long N, int* bsum, cudaStream_t st, unsigned int* err) {
+  const int nt = (int)((N + kScanTile - 1) / kScanTile);
+  HEF_CHECK_CUDA(cudaMemsetAsync(bsum, 0, (size_t)(nt == 1 ? 1 : 2 + 2 * nt) * sizeof(int), st));
+  HEF_LAUNCH("k_scan1", st, (k_scan1<In, Out><<<nt, kScanThreads, 0, st>>>(
+                                in, out, (int)N, nt, reinterpret_cast<unsigned int*>(bsum),
+                                reinterpret_cast<unsigned long long*>(bsum + 2), err)));
+  HEF_CHECK_LAUNCH();
+  return HEF_OK;
 }
 
 }  // namespace
@@ -139,13 +192,7 @@ hef_status exclusive_scan(const int* in, int* out, long long N, int* bsum, unsig
   // bsum (scan_tiles(N) + 1 ints, 8-byte aligned) holds the tile counter and,
   // for more than one tile, a 64-bit status word per kScanTile tile:
   // 2 + 2 ceil(N / 8192) ints, which then never exceeds it
-  const int nt = (int)((N + kScanTile - 1) / kScanTile);
-  HEF_CHECK_CUDA(cudaMemsetAsync(bsum, 0, (size_t)(nt == 1 ? 1 : 2 + 2 * nt) * sizeof(int), st));
-  HEF_LAUNCH("k_scan1", st, k_scan1<<<nt, kScanThreads, 0, st>>>(
-                                in, out, (int)N, nt, reinterpret_cast<unsigned int*>(bsum),
-                                reinterpret_cast<unsigned long long*>(bsum + 2), err));
-  HEF_CHECK_LAUNCH();
-  return HEF_OK;
+  return scan_with(ScanIn{in}, ScanOut{out}, N, bsum, st, err);
 }
 
 namespace {
@@ -381,14 +428,33 @@ __global__ void k_validate(int n, int m, long long P, const int64_t* __restrict_
   }
 }
 
-__global__ void k_edge_sizes(int m, const int64_t* __restrict__ eptr, const int32_t* __restrict__ sched,
-                             const unsigned int* status, int* sizes) {
-  if (status[0]) return;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < m;
-       i += (long long)gridDim.x * blockDim.x) {
-    int e = sched[i];
-    sizes[i] = (int)(eptr[e + 1] - eptr[e]);
-  }
+// x rounded to FP32 (nearest, ties to even) by integer operations in the
+// normal range: conversions share the FP64 pipe's rate of two per clock and SM.
+__device__ __forceinline__ float to_f32(double x) {
+  const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
+  const unsigned f = (h >> 20) & 0x7ffu;
+  if (f < 898u || f > 1149u) return (float)x;
+  const unsigned m = (((h & 0x7fffffffu) - (896u << 20)) << 3) | (l >> 29);
+  const unsigned rest = l & 0x1fffffffu;
+  const unsigned up = (rest > 0x10000000u || (rest == 0x10000000u && (m & 1u))) ? 1u : 0u;
+  return __uint_as_float((h & 0x80000000u) | (m + up));
+}
+
+// Reciprocals of small integers, filled by every CTA that divides by them.
+constexpr int kRecips = 64;
+// a / k rounded to nearest for an integer 1 <= k, by the reciprocal table: the
+// product is within two ulps, its residual exact, and the corrected quotient
+// rounds correctly (a quotient by k that is no rounding boundary lies at least
+// 2^-54 / k away from one, the correction's error is below 2^-104).  Three FP64
+// operations, one for powers of two, instead of a division's eight and its
+// special cases.
+__device__ __forceinline__ double div_small(double a, int k, const double2* recip) {
+  const int f = (__double2hiint(a) >> 20) & 0x7ff;
+  if (k >= kRecips || f < 200 || f > 2000) return a / (double)k;
+  const double2 r = recip[k];  // 1/k and -k
+  const double q0 = a * r.x;
+  if ((k & (k - 1)) == 0) return q0;
+  return fma(fma(r.y, q0, a), r.x, q0);
 }
 
 // Per internal hyperedge: pins in internal order, weights of both expansions,
@@ -401,6 +467,10 @@ __global__ void k_edge_fill(int m, int clique_mode, const int64_t* __restrict__ 
                             float* f_ew, float* f_ewh, float* f_ez, double* ec, int* deg,
                             double* part, double* totals) {
   if (status[0]) return;
+  __shared__ double2 recip[kRecips];
+  for (int q = threadIdx.x; q < kRecips; q += blockDim.x)
+    recip[q] = make_double2(q > 0 ? 1.0 / (double)q : 0.0, -(double)q);
+  __syncthreads();
   double wsum = 0.0;
   const int lane = threadIdx.x & 31;
   for (long long base = (long long)blockIdx.x * blockDim.x; base < m;
@@ -455,13 +525,13 @@ __global__ void k_edge_fill(int m, int clique_mode, const int64_t* __restrict__ 
     if (k >= 2) {
       wa = we;
       bh = clique_mode == HEF_CLIQUE_PAPER ? we / (0.5 * (double)k * (double)(k - 1))
-                                           : we / (double)(k - 1);
-      z = we / (double)k;
+                                           : div_small(we, k - 1, recip);
+      z = div_small(we, k, recip);
       wsum += we;
     }
     ew[i] = wa, ewh[i] = bh, ez[i] = z;
     ec[i] = k >= 2 ? bh * (double)(k - 1) : 0.0;  // clique degree contribution, added per incidence
-    f_ew[i] = (float)wa, f_ewh[i] = (float)bh, f_ez[i] = (float)z;
+    f_ew[i] = to_f32(wa), f_ewh[i] = to_f32(bh), f_ez[i] = to_f32(z);
   }
   double v[1] = {wsum};
   block_partials<1>(v, part);
@@ -485,24 +555,6 @@ __global__ void k_windows(int m, long long P, const int32_t* __restrict__ ceptr,
     const long long hi = e == m ? nwin : (long long)ceptr[e] / kWinSlots;
     for (long long w = lo; w <= hi && w <= nwin; ++w) win_edge[w] = (int32_t)e;
   }
-}
-
-// flags of hyperedges with more than kBigEdge pins (internal order)
-__global__ void k_big_flags(int m, const int32_t* __restrict__ ceptr, const unsigned int* status,
-                            int* flags) {
-  if (status[0]) return;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < m;
-       i += (long long)gridDim.x * blockDim.x)
-    flags[i] = (ceptr[i + 1] - ceptr[i]) > kBigEdge ? 1 : 0;
-}
-
-__global__ void k_big_scatter(int m, const int32_t* __restrict__ ceptr,
-                              const int32_t* __restrict__ pos, const unsigned int* status,
-                              int32_t* idx) {
-  if (status[0]) return;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < m;
-       i += (long long)gridDim.x * blockDim.x)
-    if ((ceptr[i + 1] - ceptr[i]) > kBigEdge) idx[pos[i]] = (int32_t)i;
 }
 
 // Stable counting sort of the indices i < N by keys[i] < nb (the locality
@@ -591,7 +643,10 @@ __global__ void k_node_scalars(int n, const int32_t* __restrict__ vptr, const in
     const int t0 = vptr[v], t1 = vptr[v + 1];
     // four incidences per round: their hyperedge ids, then their three
     // per-edge terms, each set of loads in flight together (sums in incidence
-    // order; the clique term ewh_e (|e|-1) comes precomputed per hyperedge)
+    // order; the clique term ewh_e (|e|-1) comes precomputed per hyperedge).
+    // The FP64 pipe bounds this: a warp's add takes 16 cycles of the SM's
+    // however few lanes have an incidence left (one 32-byte record per
+    // hyperedge instead of three gathers: 124 us for 113 at 1.1 M hyperedges)
     for (int t = t0; t < t1; t += 4) {
       int e[4];
 #pragma unroll
@@ -615,10 +670,10 @@ __global__ void k_node_scalars(int n, const int32_t* __restrict__ vptr, const in
     wsc[v] = ws;
     dc[v] = c;
     db[v] = b;
-    inv_dc[v] = c > 0.0 ? 1.0 / c : 0.0;
-    inv_db[v] = b > 0.0 ? 1.0 / b : 0.0;
-    f_wsc[v] = (float)ws, f_dc[v] = (float)c, f_db[v] = (float)b;
-    f_inv_dc[v] = (float)inv_dc[v], f_inv_db[v] = (float)inv_db[v];
+    const double ic = c > 0.0 ? 1.0 / c : 0.0, ib = b > 0.0 ? 1.0 / b : 0.0;
+    inv_dc[v] = ic, inv_db[v] = ib;
+    f_wsc[v] = to_f32(ws), f_dc[v] = to_f32(c), f_db[v] = to_f32(b);
+    f_inv_dc[v] = to_f32(ic), f_inv_db[v] = to_f32(ib);
     sc += c;
     sb += b;
   }
@@ -772,19 +827,18 @@ extern "C" hef_status hef_build_incidence(int64_t n, int64_t m, int64_t P, const
   // 2. locality schedule of hyperedges: stable counting sort by smallest pin
   // (bucket offsets in vptr, which the transpose fills later)
   if (m > 0) {
-    int grid = stride_grid(m);
+    int grid = stride_grid(m, 8);
     HEF_TRY(exclusive_scan(L.tmp, h->vptr, n, L.scan_bsum, L.sb.counter, st, h->status));
     HEF_TRY_CUDA(cudaMemsetAsync(L.cur, 0, sizeof(int) * (n + 1), st));
     HEF_LAUNCH("k_place", st, k_place<<<grid, kThreads, 0, st>>>(m, reinterpret_cast<const int32_t*>(L.keys),
                                                                 h->vptr, L.cur, h->status, L.place));
     HEF_TRY_CUDA(cudaGetLastError());
-    HEF_LAUNCH("k_bucket_order", st, k_bucket_order<<<stride_grid(n), kThreads, 0, st>>>(
+    HEF_LAUNCH("k_bucket_order", st, k_bucket_order<<<stride_grid(n, 8), kThreads, 0, st>>>(
                                          n, h->vptr, L.place, nullptr, h->status, L.vals, nullptr));
     HEF_TRY_CUDA(cudaGetLastError());
     // internal CSC offsets
-    HEF_LAUNCH("k_edge_sizes", st, k_edge_sizes<<<grid, kThreads, 0, st>>>((int)m, eptr, L.vals, h->status, L.tmp));
-    HEF_TRY_CUDA(cudaGetLastError());
-    HEF_TRY(exclusive_scan(L.tmp, h->ceptr, m, L.scan_bsum, L.sb.counter, st, h->status));
+    HEF_TRY(scan_with(SizesIn{eptr, L.vals, h->status}, ScanOut{h->ceptr}, m, L.scan_bsum, st,
+                      h->status));
     HEF_TRY_CUDA(cudaMemsetAsync(L.tmp, 0, sizeof(int) * (n + 1), st));
     HEF_LAUNCH("k_edge_fill", st, k_edge_fill<<<grid, kThreads, 0, st>>>((int)m, clique_mode, eptr, pins, w, L.vals, h->ceptr,
                                            h->status, h->counter, h->perm, h->cpins, h->slot_edge,
@@ -792,15 +846,10 @@ extern "C" hef_status hef_build_incidence(int64_t n, int64_t m, int64_t P, const
                                            L.part, h->totals));
     HEF_TRY_CUDA(cudaGetLastError());
     // list of large hyperedges (scored by whole CTAs)
-    HEF_LAUNCH("k_big_flags", st, k_big_flags<<<grid, kThreads, 0, st>>>((int)m, h->ceptr, h->status,
-                                                                        h->big_pos));
-    HEF_TRY_CUDA(cudaGetLastError());
-    HEF_TRY(exclusive_scan(h->big_pos, h->big_pos, m, L.scan_bsum, L.sb.counter, st, h->status));
+    HEF_TRY(scan_with(BigIn{h->ceptr, h->status}, BigOut{h->big_pos, h->big_idx}, m, L.scan_bsum,
+                      st, h->status));
     HEF_LAUNCH("k_windows", st, k_windows<<<stride_grid(m + 1), kThreads, 0, st>>>(
                                     (int)m, P, h->ceptr, h->status, h->win_edge));
-    HEF_TRY_CUDA(cudaGetLastError());
-    HEF_LAUNCH("k_big_scatter", st, k_big_scatter<<<grid, kThreads, 0, st>>>(
-                                        (int)m, h->ceptr, h->big_pos, h->status, h->big_idx));
     HEF_TRY_CUDA(cudaGetLastError());
   } else {
     HEF_TRY_CUDA(cudaMemsetAsync(h->ceptr, 0, sizeof(int32_t), st));
@@ -812,12 +861,12 @@ extern "C" hef_status hef_build_incidence(int64_t n, int64_t m, int64_t P, const
   // vertex (the degree counts of k_edge_fill, scanned, are the offsets)
   HEF_TRY(exclusive_scan(L.tmp, h->vptr, n, L.scan_bsum, L.sb.counter, st, h->status));
   if (P > 0) {
-    int grid = stride_grid(P);
+    int grid = stride_grid(P, 8);
     HEF_TRY_CUDA(cudaMemsetAsync(L.cur, 0, sizeof(int) * (n + 1), st));
     HEF_LAUNCH("k_place", st, k_place<<<grid, kThreads, 0, st>>>(P, h->cpins, h->vptr, L.cur, h->status,
                                                                 L.place));
     HEF_TRY_CUDA(cudaGetLastError());
-    HEF_LAUNCH("k_bucket_order", st, k_bucket_order<<<stride_grid(n), kThreads, 0, st>>>(
+    HEF_LAUNCH("k_bucket_order", st, k_bucket_order<<<stride_grid(n, 8), kThreads, 0, st>>>(
                                          n, h->vptr, L.place, h->slot_edge, h->status, h->vslot, h->vedge));
     HEF_TRY_CUDA(cudaGetLastError());
   }
