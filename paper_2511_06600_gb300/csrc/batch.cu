@@ -237,6 +237,10 @@ hef_status run_batch(const hef_batch_item* items, int G, int k, int S, int dtype
     off[g + 1] = off[g] + item_bytes(zs[g]);
   }
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost[a] > cost[b]; });
+  struct Overlap {  // items overlap on the GPU until the call returns
+    Overlap() { ortho_allow_grid(false); }
+    ~Overlap() { ortho_allow_grid(true); }
+  } overlap;
   if (t_batch_form == 1)
     return run_batch_one_launch(items, G, k, S, dtype, clique_mode, sched, ns, base, off, zs, order,
                                 cost, pool, stream);

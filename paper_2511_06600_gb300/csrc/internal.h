@@ -211,6 +211,11 @@ hef_status radix_sort(uint32_t* keys, int32_t* vals, long long N, int bits, Sort
 // turn it off.
 void krylov_allow_persistent(bool on);
 
+// Whether hef_orthonormalize calls from this thread may factor on the whole
+// grid in a cooperative launch (default on): off while a batch's items overlap,
+// whose launches could not all be resident.
+void ortho_allow_grid(bool on);
+
 // The batched form's Krylov stage: per hypergraph, the starts on its own
 // stream (krylov_batch_start, workspace as for hef_krylov_basis); then all
 // k steps of every hypergraph in cooperative launches of up to 64

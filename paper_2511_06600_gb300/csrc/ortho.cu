@@ -24,6 +24,8 @@
 //                 column blocks last to first (a column is overwritten only
 //                 after every later column has used it), 4 x 8 outputs per
 //                 thread.
+#include <algorithm>
+
 #include "internal.h"
 
 namespace hef {
@@ -349,6 +351,189 @@ __global__ void __launch_bounds__(THREADS) k_chol_aug(const double* __restrict__
     for (int j = 0; j < K; ++j) r += o.kept[j];
     *o.rank = r;
     if (fast) o.flag[0] = near_def;
+  }
+}
+
+// The same elimination by the whole grid (a cooperative launch), for matrices
+// that one SM takes long over: FP64, whose K^3 multiply-adds run at two per
+// clock and SM (0.76 ms at K = 160), and FP32 with K > kPanelMaxK, whose [A | I]
+// leaves shared memory (1.2 ms at K = 384).  Column q of [A | I] lives in the
+// shared memory of CTA q mod G (the live columns, a window that slides from the
+// left half into the right one, are then spread evenly).  Per panel of kPB
+// pivots:
+//  (a) every CTA eliminates the panel's diagonal block (in registers of warp 0,
+//      lane = column) and so holds R11, its reciprocal diagonal and the kept
+//      flags, the same bits everywhere;
+//  (b) one thread per live column runs the panel's kPB eliminations down its
+//      column (the operations of k_chol_aug in its order) and publishes the
+//      panel rows; grid barrier;
+//  (c) every CTA reads the panel rows' left part, the multipliers, and updates
+//      the rows below in its columns; the owners publish the next diagonal
+//      block; grid barrier.
+// Two barriers of about 2 us and the block's serial chain (FP64 5 us, FP32 1 us)
+// per panel are what remains: FP64 K = 160 763 -> 287 us, FP32 K = 384
+// 1210 -> 453 us.
+constexpr int kGridThreads = 256;
+constexpr int kGridMinK = 48;  // FP64: below, one CTA takes less than the barriers
+// Whether this thread's calls may take the whole grid (ortho_allow_grid).
+thread_local bool t_grid = true;
+
+struct CholGrid {
+  void* panel;            // kPB x K multipliers of the current panel
+  void* diag;             // kPB x kPB next diagonal block
+  unsigned int* arrived;  // barrier counter, zero before the launch
+  int* err;               // set when a bounded wait ran out
+};
+
+template <typename C>
+__host__ __device__ inline size_t chol_grid_smem(int K, int G) {
+  return ((size_t)((2 * K + G - 1) / G) * K + (size_t)kPB * K) * sizeof(C);
+}
+
+template <typename C, typename T>
+__global__ void __launch_bounds__(kGridThreads, 1)
+    k_chol_grid(const double* __restrict__ G, const double* __restrict__ c, const C* __restrict__ A,
+                int K, int Kp, double n, double tol, int fast, CholGrid x, CholOut o) {
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  __shared__ C R11[kPB][kPB], pinv[kPB];  // R11[p][i]: row p, column i of the panel
+  __shared__ int kept[512], alive;
+  const int tid = threadIdx.x, lane = tid & 31, nb = gridDim.x, b = blockIdx.x;
+  const int ncol = (2 * K - b + nb - 1) / nb;  // own columns q = b + nb cc
+  C* S = reinterpret_cast<C*>(sm_raw);         // column cc: K rows at S + cc K
+  C* M = S + (size_t)((2 * K + nb - 1) / nb) * K;  // kPB x K
+  C* panel = static_cast<C*>(x.panel);
+  C* diag = static_cast<C*>(x.diag);
+  for (int e = tid; e < ncol * K; e += kGridThreads) {
+    const int q = b + nb * (e / K), i = e % K;
+    S[e] = q < K ? A[(size_t)q * K + i] : (q - K == i ? (C)1 : (C)0);  // A is symmetric
+  }
+  if (tid == 0) alive = 1;
+  __syncthreads();
+  unsigned int want = 0;
+  auto grid_sync = [&]() -> bool {
+    want += (unsigned)nb;
+    __syncthreads();
+    if (tid == 0) {
+      __threadfence();
+      atomicAdd(x.arrived, 1u);
+      unsigned int it = 0;
+      while (*reinterpret_cast<volatile unsigned int*>(x.arrived) < want) {
+        if (++it > (1u << 21) || *reinterpret_cast<volatile int*>(x.err)) {
+          atomicExch(x.err, 1);
+          alive = 0;
+          break;
+        }
+      }
+      __threadfence();
+    }
+    __syncthreads();
+    return alive != 0;
+  };
+  int near_def = 0;
+  bool ok = true;
+  for (int j0 = 0; j0 < K && ok; j0 += kPB) {
+    const int np = min(kPB, K - j0), jend = j0 + np;
+    // (a)
+    if (tid < 32) {
+      const int col = lane & (kPB - 1);
+      C v[kPB];
+#pragma unroll
+      for (int r = 0; r < kPB; ++r)
+        v[r] = (r < np && col < np) ? (j0 == 0 ? A[(size_t)r * K + col] : __ldcg(diag + r * kPB + col)) : (C)0;
+      const double gj = j0 + col < K ? G[(size_t)(j0 + col) * (K + 1)] : 0.0;
+      const C ref = (C)gj, thr_keep = (C)(tol * gj), thr_near = (C)(1e-4 * gj);
+#pragma unroll
+      for (int p = 0; p < kPB; ++p) {
+        if (p < np) {  // warp-uniform
+          const C d = __shfl_sync(0xffffffffu, v[p], p);
+          const C rf = __shfl_sync(0xffffffffu, ref, p), tk = __shfl_sync(0xffffffffu, thr_keep, p);
+          const C tn = __shfl_sync(0xffffffffu, thr_near, p);
+          const bool kj = rf > (C)0 && d > tk;
+          near_def |= (fast && kj && d <= tn) ? 1 : 0;
+          const C pv = kj ? rsqrt(d) : (C)0;
+          v[p] = kj ? v[p] * pv : (C)0;
+#pragma unroll
+          for (int i = p + 1; i < kPB; ++i) {
+            const C r = __shfl_sync(0xffffffffu, v[p], i);
+            if (kj) v[i] -= r * v[p];
+          }
+          if (lane == 0) pinv[p] = pv, kept[j0 + p] = kj;
+        }
+      }
+      if (lane < kPB)
+#pragma unroll
+        for (int r = 0; r < kPB; ++r) R11[r][col] = v[r];
+    }
+    __syncthreads();
+    // (b) live columns [j0, K + jend): the panel's eliminations down the column
+    for (int cc = tid; cc < ncol; cc += kGridThreads) {
+      const int q = b + nb * cc;
+      if (q < j0 || q >= K + jend) continue;
+      C* col = S + (size_t)cc * K + j0;
+      C y[kPB];
+#pragma unroll
+      for (int p = 0; p < kPB; ++p) y[p] = p < np ? col[p] : (C)0;
+#pragma unroll
+      for (int p = 0; p < kPB; ++p) {
+        if (p < np) {
+          y[p] = kept[j0 + p] ? y[p] * pinv[p] : (C)0;
+#pragma unroll
+          for (int i = p + 1; i < kPB; ++i)
+            if (i < np) y[i] -= R11[p][i] * y[p];
+        }
+      }
+#pragma unroll
+      for (int p = 0; p < kPB; ++p)
+        if (p < np) {
+          col[p] = y[p];
+          if (q < K) panel[(size_t)p * K + q] = y[p];
+        }
+    }
+    if (jend >= K) break;  // nothing below the last panel
+    if (!(ok = grid_sync())) break;
+    // (c)
+    for (int e = tid; e < np * (K - jend); e += kGridThreads) {
+      const int p = e / (K - jend), i = jend + e % (K - jend);
+      M[p * K + i] = __ldcg(panel + (size_t)p * K + i);
+    }
+    __syncthreads();
+    const int rows = K - jend, c0 = max(0, (jend - b + nb - 1) / nb);  // first own column >= jend
+    const int c1 = min(ncol, (K + jend - b + nb - 1) / nb);
+    for (int e = tid; e < (c1 - c0) * rows; e += kGridThreads) {
+      const int cc = c0 + e / rows, i = jend + e % rows;
+      C* col = S + (size_t)cc * K;
+      C acc = col[i];
+#pragma unroll
+      for (int p = 0; p < kPB; ++p)
+        if (p < np) acc -= M[p * K + i] * col[j0 + p];
+      col[i] = acc;
+      const int q = b + nb * cc;
+      if (q < min(jend + kPB, K) && i < jend + kPB) diag[(i - jend) * kPB + (q - jend)] = acc;
+    }
+    ok = grid_sync();
+  }
+  if (!ok) return;
+  __syncthreads();
+  // outputs from the own columns: R's column i (FP64), R^-1's row i = column
+  // K + i of the right half; CTA 0 the vectors, the padding and the counts
+  T* Rinv = static_cast<T*>(o.Rinv);
+  T* mu = static_cast<T*>(o.mu);
+  for (int e = tid; e < ncol * Kp; e += kGridThreads) {
+    const int q = b + nb * (e / Kp), j = e % Kp;
+    const C* col = S + (size_t)(e / Kp) * K;
+    if (q >= K) Rinv[(size_t)(q - K) * Kp + j] = j < K && q - K <= j ? (T)col[j] : (T)0;
+    else if (o.R && j < K) o.R[(size_t)j * K + q] = j <= q ? (double)col[j] : 0.0;
+  }
+  if (b == 0) {
+    for (int e = tid; e < (Kp - K) * Kp; e += kGridThreads) Rinv[(size_t)K * Kp + e] = (T)0;
+    for (int i = tid; i < Kp; i += kGridThreads) mu[i] = i < K ? (T)(c[i] / n) : (T)0;
+    for (int i = tid; i < K; i += kGridThreads) o.kept[i] = kept[i];
+    if (tid == 0) {
+      int r = 0;
+      for (int j = 0; j < K; ++j) r += kept[j];
+      *o.rank = r;
+      if (fast) o.flag[0] = near_def;
+    }
   }
 }
 
@@ -813,13 +998,10 @@ hef_status run_ortho(long long n, int K, T* V, long long ldv, double* R_out, int
   HEF_ENSURE_SMEM(k_apply<T>, (int)apply_smem(RB));
   const int agrid = (int)((n + RB - 1) / RB);
   const int athreads = RB * 2;  // (RB / 4) row groups x 8 column groups
-  // FP32 form: the FP32 elimination works in shared memory when [A | I]
-  // fits (K <= 160), else in the (L2-resident) FP64 scratch reused as FP32
-  const size_t fast_smem = (size_t)K * 2 * K * sizeof(float);
+  // FP32 form: the FP32 elimination works in one CTA's shared memory when
+  // [A | I] fits (K <= 160), else over the grid
   const bool fast_ok = sizeof(T) == 4;
-  const bool fast_in_smem = fast_ok && fast_smem <= 200 * 1024;
   const bool panels = fast_ok && panel_supported(K);
-  if (fast_in_smem) HEF_ENSURE_SMEM((k_chol_aug<float, T>), fast_smem);
   if (panels) HEF_ENSURE_SMEM(k_chol_panels<T>, panel_smem(K));
   const double tol = sizeof(T) == 8 ? 1e-12 : 1e-5;
   // second pass: the first-order factor of the near-identity Gram is exact to
@@ -856,21 +1038,46 @@ hef_status run_ortho(long long n, int K, T* V, long long ldv, double* R_out, int
       if (!want_R) o.R = nullptr;
       HEF_LAUNCH("k_gram_project", st, k_gram_project<<<stride_grid((long long)K * K, 2), kThreads, 0,
                                                          st>>>(w.G, w.c, K, (double)n, w.A64, w.A32));
+      // the factorisation by one CTA in shared memory, or by the grid where one
+      // SM's arithmetic (FP64) or shared memory (FP32) does not do and no other
+      // work of the caller's shares the GPU
+      auto on_grid = [&](auto zero, const auto* A, int fast) -> hef_status {
+        using C = decltype(zero);
+        // about two (FP64) or eight (FP32) live columns per CTA
+        const int ctas = std::min(num_sms(), std::max(1, (K + kPB) / (sizeof(C) == 8 ? 2 : 8)));
+        const size_t smem = chol_grid_smem<C>(K, ctas);
+        HEF_ENSURE_SMEM((k_chol_grid<C, T>), smem);
+        CholGrid x{w.Wg, w.Wg + (size_t)kPB * K, reinterpret_cast<unsigned int*>(w.flag + 2), w.flag + 1};
+        cudaError_t e = cudaSuccess;
+        HEF_LAUNCH("k_chol_grid", st,
+                   e = launch_cooperative_smem(k_chol_grid<C, T>, ctas, kGridThreads, smem, st,
+                                               (const double*)w.G, (const double*)w.c, A, K, Kp,
+                                               (double)n, tol, fast, x, o));
+        if (e != cudaSuccess) return set_error(HEF_ERR_CUDA, "k_chol_grid: %s", cudaGetErrorString(e));
+        return HEF_OK;
+      };
       if (fast_ok) {
         if (panels) {
           HEF_LAUNCH("k_chol_panels", st, k_chol_panels<T><<<1, kPanelThreads, panel_smem(K), st>>>(
                                               w.G, w.c, w.A32, K, Kp, (double)n, tol, o));
+        } else if (t_grid) {
+          hef_status s = on_grid(0.0f, (const float*)w.A32, 1);
+          if (s) return s;
         } else {
-          HEF_LAUNCH("k_chol_aug", st, k_chol_aug<float, T><<<1, 1024, fast_in_smem ? fast_smem : 0, st>>>(
+          HEF_LAUNCH("k_chol_aug", st, k_chol_aug<float, T><<<1, 1024, 0, st>>>(
                                            w.G, w.c, w.A32, K, Kp, (double)n, tol,
-                                           fast_in_smem ? nullptr : reinterpret_cast<float*>(w.Wg),
-                                           fast_in_smem ? 1 : 0, 1, 0, o));
+                                           reinterpret_cast<float*>(w.Wg), 0, 1, 0, o));
         }
       }
       // exact FP64 path: always for the FP64 form, on demand for the FP32 form
-      HEF_LAUNCH("k_chol_aug", st, k_chol_aug<double, T><<<1, 1024, 0, st>>>(
-                                       w.G, w.c, w.A64, K, Kp, (double)n, tol, w.Wg, 0, 0,
-                                       fast_ok ? 0 : 1, o));
+      if (!fast_ok && K >= kGridMinK && t_grid) {
+        hef_status s = on_grid(0.0, (const double*)w.A64, 0);
+        if (s) return s;
+      } else {
+        HEF_LAUNCH("k_chol_aug", st, k_chol_aug<double, T><<<1, 1024, 0, st>>>(
+                                         w.G, w.c, w.A64, K, Kp, (double)n, tol, w.Wg, 0, 0,
+                                         fast_ok ? 0 : 1, o));
+      }
     } else {
       HEF_CHECK_CUDA(cudaMemsetAsync(w.flag, 0, sizeof(int), st));  // flag[0] only
       HEF_LAUNCH("k_chol_series", st, k_chol_series<T><<<stride_grid((long long)Kp * Kp, 2),
@@ -912,6 +1119,8 @@ hef_status run_ortho(long long n, int K, T* V, long long ldv, double* R_out, int
 }
 
 }  // namespace
+
+void ortho_allow_grid(bool on) { t_grid = on; }
 
 }  // namespace hef
 

@@ -51,3 +51,40 @@ def test_one_long_hyperedge():
                                               for e in range(H.m)])
     a, b = both(H, 4, 2, torch.float64)
     assert rel_errors(a, b)["normwise"] <= 1e-12
+
+
+def test_calls_on_several_streams_at_once():
+    # cooperative launches of different streams and threads take turns
+    import threading
+
+    import paper_2511_06600_gb300 as hef
+    from tests._gpu import to_dev
+    nets = []
+    for i in range(4):
+        H = grid_netlist(40 + 9 * i, 50, int(1.05 * (40 + 9 * i) * 50), i)
+        nets.append((H, to_dev(H, *start_block(H.n, H.m, 2, i))))
+
+    def score(H, t):
+        return hef.hyperedge_resistance(H.n, t["eptr"], t["pins"], t["w"], t["x0c"], t["x0b"], 12,
+                                        torch.float64)["R"]
+
+    alone = [score(H, t).cpu() for H, t in nets]
+    torch.cuda.synchronize()
+    got, errors = [None] * 4, []
+
+    def work(i):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(5):
+                    got[i] = score(*nets[i]).cpu()
+        except Exception as e:  # noqa: BLE001
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(4)]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    assert not errors
+    for a, b in zip(alone, got):
+        assert torch.equal(a, b)

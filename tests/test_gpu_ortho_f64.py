@@ -97,3 +97,32 @@ def test_repeatable_and_independent_of_the_stream():
     with torch.cuda.stream(torch.cuda.Stream()):
         b = run(V)
     assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+
+
+@pytest.mark.parametrize("dtype,K", [(torch.float64, 47), (torch.float64, 48), (torch.float64, 63),
+                                     (torch.float64, 150), (torch.float64, 400),
+                                     (torch.float32, 161), (torch.float32, 200),
+                                     (torch.float32, 384), (torch.float32, 511)])
+def test_elimination_over_the_grid(dtype, K):
+    # K around the sizes at which the elimination moves to the grid, partial
+    # panels, and dependent columns whose pivots must be dropped; the rank and
+    # the orthogonality to 8 (K + 8) eps (FP32: the second pass leaves rounding
+    # of the FP32 basis and of its tensor-core sums, 64 K eps)
+    import paper_2511_06600_gb300 as hef
+    rng = np.random.default_rng(K)
+    n = 6 * K + 11
+    V = rng.standard_normal((n, K))
+    V[:, K // 2] = V[:, 1] + V[:, 3]
+    V[:, K - 1] = 0
+    d = torch.zeros(n, hef.padded_ld(K, dtype), dtype=dtype, device=DEV)
+    d[:, :K] = torch.from_numpy(V).to(DEV)
+    Q, R, rank = hef.orthonormalize(d, K, want_R=True)
+    Q = Q[:, :K].double().cpu().numpy()
+    assert int(rank) == K - 2
+    assert (Q[:, K // 2] == 0).all() and (Q[:, K - 1] == 0).all()
+    keep = [c for c in range(K) if c not in (K // 2, K - 1)]
+    tol = 8 * (K + 8) * EPS if dtype == torch.float64 else 64 * K * np.finfo(np.float32).eps
+    assert np.abs(Q[:, keep].T @ Q[:, keep] - np.eye(K - 2)).max() <= tol
+    A = V - V.mean(0)
+    res = np.abs(A - Q @ R.cpu().numpy()).max(0)
+    assert (res[keep] <= tol * np.abs(V).max() * np.sqrt(K)).all()
