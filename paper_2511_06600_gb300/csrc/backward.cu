@@ -93,10 +93,15 @@ __global__ void __launch_bounds__(256) k_bwd_scores(IncView g, const T* __restri
   for (long long e = warp; e < g.m; e += nwarps) {
     const int a = g.ceptr[e], b = g.ceptr[e + 1];
     if (b - a < 2) continue;
+    using Ord = Order<T>;  // FP64 values compared as integers
+    typename Ord::Key kx[NC], kn[NC];
     T mx[NC], mn[NC];
     int imx[NC], imn[NC];
 #pragma unroll
-    for (int c = 0; c < NC; ++c) mx[c] = lowest_v<T>(), mn[c] = -lowest_v<T>(), imx[c] = a, imn[c] = a;
+    for (int c = 0; c < NC; ++c) {
+      mx[c] = lowest_v<T>(), mn[c] = -lowest_v<T>(), imx[c] = a, imn[c] = a;
+      kx[c] = Ord::key(mx[c]), kn[c] = Ord::key(mn[c]);
+    }
     for (int t = a; t < b; ++t) {
       const T* row = Q + (long long)dbg_index(g.cpins[t], g.n, g.status) * ldq;
 #pragma unroll
@@ -104,8 +109,10 @@ __global__ void __launch_bounds__(256) k_bwd_scores(IncView g, const T* __restri
         const int col = lane + 32 * c;
         if (col < K) {
           const T v = row[col];
-          if (v > mx[c]) mx[c] = v, imx[c] = t;
-          if (v < mn[c]) mn[c] = v, imn[c] = t;
+          const typename Ord::Key k = Ord::key(v);
+          const bool num = Ord::number(v);
+          if (num && k > kx[c]) kx[c] = k, mx[c] = v, imx[c] = t;
+          if (num && k < kn[c]) kn[c] = k, mn[c] = v, imn[c] = t;
         }
       }
     }
@@ -117,7 +124,7 @@ __global__ void __launch_bounds__(256) k_bwd_scores(IncView g, const T* __restri
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
       const int col = lane + 32 * c;
-      if (iq[c] != 0.0) {
+      if (!Order<double>::zero(iq[c])) {
         const double sp = (double)mx[c] - (double)mn[c];
         double sb = 2.0 * qhb[c] * we * sp;
         if (col == istar) sb += 2.0 * ge * sp * iq[c];

@@ -365,6 +365,30 @@ __device__ __forceinline__ DFloat df_add(DFloat a, DFloat b) {
   return {h, __fsub_rn(e, __fsub_rn(h, s))};
 }
 
+// Comparisons of basis values without the FP64 pipe (two per clock and SM):
+// Order<T>::key(x) orders like x (-0 as +0) and number(x) is false for NaN, for
+// which every comparison is false.  FP32 values are their own keys.
+template <typename T>
+struct Order {
+  using Key = T;
+  static __device__ __forceinline__ Key key(T x) { return x; }
+  static __device__ __forceinline__ bool number(T x) { return x == x; }
+  static __device__ __forceinline__ bool zero(T x) { return x == (T)0; }
+};
+template <>
+struct Order<double> {
+  using Key = long long;
+  static __device__ __forceinline__ Key key(double x) {
+    long long b = __double_as_longlong(x);
+    b = (b << 1) == 0 ? 0 : b;
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+  }
+  static __device__ __forceinline__ bool number(double x) {
+    return ((__double2hiint(x) & 0x7fffffff) | (__double2loint(x) != 0 ? 1 : 0)) <= 0x7ff00000;
+  }
+  static __device__ __forceinline__ bool zero(double x) { return (__double_as_longlong(x) << 1) == 0; }
+};
+
 inline int red_groups(int nblk) { return (nblk + kRedGroup - 1) / kRedGroup; }
 
 // In one CTA: out[slot] = sum over b < nblk of part[b * nslot + slot], for

@@ -71,10 +71,8 @@ struct Extrema<double> {
     mx = key(__double_as_longlong(lowest<double>())), mn = key(__double_as_longlong(-lowest<double>()));
   }
   __device__ __forceinline__ void add(double x) {
-    const int hi = __double2hiint(x);
-    const bool number = ((hi & 0x7fffffff) | (__double2loint(x) != 0 ? 1 : 0)) <= 0x7ff00000;
     const long long k = key(__double_as_longlong(x));
-    if (number) mx = max(mx, k), mn = min(mn, k);
+    if (Order<double>::number(x)) mx = max(mx, k), mn = min(mn, k);
   }
   __device__ __forceinline__ double spread() const {
     return __longlong_as_double(key(mx)) - __longlong_as_double(key(mn));
@@ -938,7 +936,8 @@ __global__ void __launch_bounds__(256) k_score_ratio(IncView g, const T* __restr
 // scan of the whole row.  The routing pins: the lanes split the hyperedge's
 // pins the same way and combine the extrema of the arg-max column by value,
 // then position.  R_e, the arg-max column and the routing pins are therefore
-// bit-identical to k_score_ratio's.
+// bit-identical to k_score_ratio's.  FP64 values are compared as integers: the
+// comparisons were most of this kernel's time on the FP64 pipe.
 constexpr int kRatioLanes = 8;
 
 template <typename T>
@@ -949,6 +948,8 @@ __global__ void __launch_bounds__(256) k_score_ratio8(IncView g, const T* __rest
                                                       double* R_out, int32_t* argvec, int32_t* pmax,
                                                       int32_t* pmin) {
   if (g.status[0]) return;
+  using Ord = Order<T>;
+  using Key = typename Ord::Key;
   constexpr int V = 16 / sizeof(T);  // elements per 16-byte chunk
   constexpr int U = 4;               // chunks of a lane in flight
   extern __shared__ unsigned char iq_raw[];
@@ -966,7 +967,8 @@ __global__ void __launch_bounds__(256) k_score_ratio8(IncView g, const T* __rest
     int a = 0, b = 0;
     if (valid) a = g.ceptr[e], b = g.ceptr[e + 1];
     const bool scored = valid && b - a >= 2;
-    T best = (T)-1, spb = 0;
+    Key best = Ord::key((T)-1);
+    T spb = 0;
     int bcol = -1;
     if (scored) {
       const uint4* row = reinterpret_cast<const uint4*>(spread + e * ldsp);
@@ -983,33 +985,39 @@ __global__ void __launch_bounds__(256) k_score_ratio8(IncView g, const T* __rest
 #pragma unroll
           for (int q = 0; q < V; ++q) {
             const int i = (c0 + u * kRatioLanes) * V + q;
-            if (i >= K || iq[i] == (T)0) continue;
+            if (i >= K || Ord::zero(iq[i])) continue;
             const T r = sp[u][q] * sp[u][q] * iq[i];
-            if (r > best) best = r, bcol = i, spb = sp[u][q];
+            const Key k = Ord::key(r);
+            if (Ord::number(r) && k > best) best = k, bcol = i, spb = sp[u][q];
           }
       }
     }
     // combine the group's candidates: larger ratio, then lower column
 #pragma unroll
     for (int o = kRatioLanes / 2; o > 0; o >>= 1) {
-      const T ob = __shfl_xor_sync(0xffffffffu, best, o);
+      const Key ob = __shfl_xor_sync(0xffffffffu, best, o);
       const T os = __shfl_xor_sync(0xffffffffu, spb, o);
       const int oc = __shfl_xor_sync(0xffffffffu, bcol, o);
       if (oc >= 0 && (bcol < 0 || ob > best || (ob == best && oc < bcol))) best = ob, bcol = oc, spb = os;
     }
     const bool any = scored && bcol >= 0;
-    T vmax = lowest<T>(), vmin = -lowest<T>();
+    const Key low = Ord::key(lowest<T>()), high = Ord::key(-lowest<T>());
+    Key vmax = low, vmin = high;
     int tmax = INT_MAX, tmin = INT_MAX;
     if (any && (pmax || pmin)) {
       for (int t = a + sub; t < b; t += kRatioLanes) {
         const T v = qw<T>(Q[(long long)dbg_index(g.cpins[t], g.n, g.status) * ldq + bcol]);
-        if (tmax == INT_MAX || v > vmax) vmax = v, tmax = t;
-        if (tmin == INT_MAX || v < vmin) vmin = v, tmin = t;
+        // a NaN loses to every number (as in the spreads), but keeps its place
+        // when there is none
+        const bool num = Ord::number(v);
+        const Key kx = num ? Ord::key(v) : low, kn = num ? Ord::key(v) : high;
+        if (tmax == INT_MAX || kx > vmax) vmax = kx, tmax = t;
+        if (tmin == INT_MAX || kn < vmin) vmin = kn, tmin = t;
       }
     }
 #pragma unroll
     for (int o = kRatioLanes / 2; o > 0; o >>= 1) {
-      const T ovx = __shfl_xor_sync(0xffffffffu, vmax, o), ovn = __shfl_xor_sync(0xffffffffu, vmin, o);
+      const Key ovx = __shfl_xor_sync(0xffffffffu, vmax, o), ovn = __shfl_xor_sync(0xffffffffu, vmin, o);
       const int otx = __shfl_xor_sync(0xffffffffu, tmax, o), otn = __shfl_xor_sync(0xffffffffu, tmin, o);
       if (otx != INT_MAX && (tmax == INT_MAX || ovx > vmax || (ovx == vmax && otx < tmax))) vmax = ovx, tmax = otx;
       if (otn != INT_MAX && (tmin == INT_MAX || ovn < vmin || (ovn == vmin && otn < tmin))) vmin = ovn, tmin = otn;
