@@ -178,33 +178,58 @@ __global__ void __launch_bounds__(256) k_bwd_qbar(IncView g, int K, const double
 
 // ---------------------------------------------------------------- QR adjoint
 
-// part[chunk][i][j] = sum over the chunk's rows r of Qbar[r][i] * Q[r][j],
-// in the storage type within a chunk (FP32 products and sums for the FP32
-// form: FP64 runs at 1/64 of the rate) and FP64 across chunks.
+// Element idx of the lower triangle, row by row: i >= j.
+__device__ __forceinline__ void lower_of(int idx, int& i, int& j) {
+  i = (int)((sqrtf(8.0f * (float)idx + 1.0f) - 1.0f) * 0.5f);
+  while (i * (i + 1) / 2 > idx) --i;
+  while ((i + 1) * (i + 2) / 2 <= idx) ++i;
+  j = idx - i * (i + 1) / 2;
+}
+
+// part[chunk][idx] = sum over the chunk's rows r of Qbar[r][i] * Q[r][j] for
+// the elements i >= j that copyltu reads, in the storage type within a chunk
+// (FP32 products and sums for the FP32 form: FP64 runs at 1/64 of the rate) and
+// FP64 across chunks.  In FP64 bound by that pipe: 174 -> 105 us without the
+// other triangle (200,000 rows, K = 20).
 template <typename T>
 __global__ void k_bwd_xgram(const T* __restrict__ Qbar, const T* __restrict__ Q, long long ldq,
                             long long n, int K, long long rows_per_chunk, double* part) {
-  const int chunk = blockIdx.y;
+  const int chunk = blockIdx.y, L = K * (K + 1) / 2;
   const long long r0 = (long long)chunk * rows_per_chunk;
   const long long r1 = min(n, r0 + rows_per_chunk);
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < K * K; idx += gridDim.x * blockDim.x) {
-    const int i = idx / K, j = idx % K;
+  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < L; idx += gridDim.x * blockDim.x) {
+    int i, j;
+    lower_of(idx, i, j);
     T s = 0;
     for (long long r = r0; r < r1; ++r) s += Qbar[r * K + i] * Q[r * ldq + j];
-    part[(size_t)chunk * K * K + idx] = (double)s;
+    part[(size_t)chunk * L + idx] = (double)s;
   }
 }
 
 // C = copyltu(-Qbar^T Q): C[i][j] = -(Qbar^T Q)[max(i,j)][min(i,j)] (summed
-// in FP64, stored in the storage type).
+// in FP64, stored in the storage type).  A CTA takes 32 elements of the lower
+// triangle: warp w sums the chunks w, w + 8, ..., then the warps' sums are
+// added in order (one thread per element walked all chunks: 84 -> 17 us at
+// 782 chunks, K = 20).
 template <typename T>
-__global__ void k_bwd_copyltu(const double* __restrict__ part, int K, int nchunk, T* C) {
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < K * K; idx += gridDim.x * blockDim.x) {
-    const int i = idx / K, j = idx % K;
-    const int hi = i > j ? i : j, lo = i > j ? j : i;
-    double s = 0.0;
-    for (int q = 0; q < nchunk; ++q) s += part[(size_t)q * K * K + hi * K + lo];
-    C[idx] = (T)-s;
+__global__ void __launch_bounds__(256) k_bwd_copyltu(const double* __restrict__ part, int K, int nchunk,
+                                                     T* C) {
+  __shared__ double red[8][32];
+  const int L = K * (K + 1) / 2, e = threadIdx.x & 31, sub = threadIdx.x >> 5;
+  const int idx = blockIdx.x * 32 + e;
+  double s = 0.0;
+  if (idx < L) {
+#pragma unroll 4
+    for (int q = sub; q < nchunk; q += 8) s += part[(size_t)q * L + idx];
+  }
+  red[sub][e] = s;
+  __syncthreads();
+  if (sub == 0 && idx < L) {
+#pragma unroll
+    for (int w = 1; w < 8; ++w) s += red[w][e];
+    int i, j;
+    lower_of(idx, i, j);
+    C[(size_t)i * K + j] = C[(size_t)j * K + i] = (T)-s;
   }
 }
 
@@ -268,14 +293,28 @@ __global__ void k_bwd_qr_abar(const T* __restrict__ Z, const T* __restrict__ Rin
   }
 }
 
-// colsum[j] = sum_r A[r][j] (A n x K): CTA-strided rows summed in the
-// storage type, one FP64 atomic per CTA and column.
+// colsum[j] = sum_r A[r][j] (A n x K): each thread sums one column over rows in
+// the storage type, the CTA's threads of a column meet in FP64, one FP64 atomic
+// per CTA and column.  Whole rows per CTA and round (with one thread per column
+// 20 of 256 worked at K = 20: 97 -> 16 us at 200,000 rows).
 template <typename T>
-__global__ void k_bwd_colsum(const T* __restrict__ A, long long n, int K, double* colsum) {
-  for (int j = threadIdx.x; j < K; j += blockDim.x) {
-    T s = 0;
-    for (long long r = blockIdx.x; r < n; r += gridDim.x) s += A[r * K + j];
-    atomicAdd(&colsum[j], (double)s);
+__global__ void __launch_bounds__(512) k_bwd_colsum(const T* __restrict__ A, long long n, int K,
+                                                    double* colsum) {
+  __shared__ double red[512];
+  const int rpi = 512 / K;  // rows per round (K <= 512)
+  const int j = threadIdx.x % K, r0 = threadIdx.x / K;
+  T s = 0;
+  if (r0 < rpi) {
+    const long long step = (long long)gridDim.x * rpi;
+#pragma unroll 4
+    for (long long r = (long long)blockIdx.x * rpi + r0; r < n; r += step) s += A[r * K + j];
+  }
+  red[threadIdx.x] = (double)s;
+  __syncthreads();
+  if (threadIdx.x < K) {
+    double t = red[threadIdx.x];
+    for (int q = 1; q < rpi; ++q) t += red[q * K + threadIdx.x];
+    atomicAdd(&colsum[threadIdx.x], t);
   }
 }
 
@@ -724,19 +763,19 @@ hef_status run_bwd(const hef_incidence* inc, int k, int S, const double* x0c, co
 
   // 2. QR adjoint -> Abar and its column means
   const long long rpc = (n + w.nchunk - 1) / w.nchunk;
-  const int kk_blocks = (K * K + 255) / 256;
+  const int lower = K * (K + 1) / 2;
   HEF_LAUNCH("k_bwd_xgram", st,
-             k_bwd_xgram<T><<<dim3(kk_blocks, w.nchunk), 256, 0, st>>>(Qbar, Q, ldq, n, K, rpc,
+             k_bwd_xgram<T><<<dim3((lower + 255) / 256, w.nchunk), 256, 0, st>>>(Qbar, Q, ldq, n, K, rpc,
                                                                          w.part));
   HEF_LAUNCH("k_bwd_copyltu", st,
-             k_bwd_copyltu<T><<<kk_blocks, 256, 0, st>>>(w.part, K, w.nchunk, Ct));
+             k_bwd_copyltu<T><<<(lower + 31) / 32, 256, 0, st>>>(w.part, K, w.nchunk, Ct));
   HEF_LAUNCH("k_bwd_rinv", st, k_bwd_rinv<T><<<1, 1024, 0, st>>>(Rfac, K, w.Rinv, RinvT));
   const int eg = stride_grid(n * K, 8);
   HEF_LAUNCH("k_bwd_qr_z", st, k_bwd_qr_z<T><<<eg, kThreads, 0, st>>>(Q, ldq, Qbar, Ct, n, K, Z));
   HEF_LAUNCH("k_bwd_qr_abar", st, k_bwd_qr_abar<T><<<eg, kThreads, 0, st>>>(Z, RinvT, n, K, Abar));
   HEF_CHECK_CUDA(cudaMemsetAsync(w.colsum, 0, K * sizeof(double), st));
   HEF_LAUNCH("k_bwd_colsum", st,
-             k_bwd_colsum<T><<<num_sms() * 2, 256, 0, st>>>(Abar, n, K, w.colsum));
+             k_bwd_colsum<T><<<num_sms() * 2, 512, 0, st>>>(Abar, n, K, w.colsum));
   HEF_LAUNCH("k_bwd_mean", st, k_bwd_mean<T><<<1, 256, 0, st>>>(w.colsum, n, K, mean));
   HEF_CHECK_LAUNCH();
 
