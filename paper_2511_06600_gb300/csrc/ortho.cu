@@ -370,9 +370,9 @@ __global__ void __launch_bounds__(THREADS) k_chol_aug(const double* __restrict__
 //  (c) every CTA reads the panel rows' left part, the multipliers, and updates
 //      the rows below in its columns; the owners publish the next diagonal
 //      block; grid barrier.
-// Two barriers of about 2 us and the block's serial chain (FP64 5 us, FP32 1 us)
-// per panel are what remains: FP64 K = 160 763 -> 287 us, FP32 K = 384
-// 1210 -> 453 us.
+// The diagonal block's serial chain, the columns' and two barriers, 28 us (FP64)
+// or 19 us (FP32) per panel, are what remains: FP64 K = 160 763 -> 287 us, FP32
+// K = 384 1210 -> 453 us.
 constexpr int kGridThreads = 256;
 constexpr int kGridMinK = 48;  // FP64: below, one CTA takes less than the barriers
 // Whether this thread's calls may take the whole grid (ortho_allow_grid).
