@@ -237,21 +237,20 @@ hef_status run_batch(const hef_batch_item* items, int G, int k, int S, int dtype
     off[g + 1] = off[g] + item_bytes(zs[g]);
   }
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost[a] > cost[b]; });
-  struct Overlap {  // items overlap on the GPU until the call returns
-    Overlap() { ortho_allow_grid(false); }
-    ~Overlap() { ortho_allow_grid(true); }
+  // items overlap on the GPU: grids with barriers of their own could not all
+  // be resident (the thread's own settings come back when the call returns)
+  struct Overlap {
+    bool grid = ortho_allow_grid(false), persistent = krylov_allow_persistent(false);
+    ~Overlap() { ortho_allow_grid(grid), krylov_allow_persistent(persistent); }
   } overlap;
   if (t_batch_form == 1)
     return run_batch_one_launch(items, G, k, S, dtype, clique_mode, sched, ns, base, off, zs, order,
                                 cost, pool, stream);
-  // items overlap on the GPU: one-launch Krylov grids could not all be resident
-  krylov_allow_persistent(false);
   for (int g : order) {
     const int si = sched[g];
     hef_status r = run_item(items[g], k, S, dtype, clique_mode, zs[g], base + off[g], pool->s[si]);
     if (r && !first) first = r;
   }
-  krylov_allow_persistent(true);
   // join every stream that took part, also after an error (a capture must
   // end with all forked streams joined)
   for (int i = 0; i < ns; ++i) {

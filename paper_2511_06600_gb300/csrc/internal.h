@@ -208,13 +208,13 @@ hef_status radix_sort(uint32_t* keys, int32_t* vals, long long N, int bits, Sort
 // Whether hef_krylov_basis(_tape) calls from this thread may run all Krylov
 // steps as one persistent launch (default on).  The persistent grid needs
 // every CTA resident at once, so callers that overlap other work on the GPU
-// turn it off.
-void krylov_allow_persistent(bool on);
+// turn it off.  Returns the setting it replaces, for the caller to put back.
+bool krylov_allow_persistent(bool on);
 
 // Whether hef_orthonormalize calls from this thread may factor on the whole
 // grid in a cooperative launch (default on): off while a batch's items overlap,
-// whose launches could not all be resident.
-void ortho_allow_grid(bool on);
+// whose launches could not all be resident.  Returns the setting it replaces.
+bool ortho_allow_grid(bool on);
 
 // The batched form's Krylov stage: per hypergraph, the starts on its own
 // stream (krylov_batch_start, workspace as for hef_krylov_basis); then all

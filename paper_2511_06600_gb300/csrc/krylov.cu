@@ -1694,7 +1694,7 @@ hef_status krylov_batch_steps(const KrylovBatchArg* items, int G, int k, int S, 
   return batch_steps<float, float>(items, G, k, S, st);
 }
 
-void krylov_allow_persistent(bool on) { t_persistent = on; }
+bool krylov_allow_persistent(bool on) { return std::exchange(t_persistent, on); }
 void krylov_force_oversized(bool on) { t_force_oversized = on; }
 
 }  // namespace hef

@@ -25,6 +25,7 @@
 //                 after every later column has used it), 4 x 8 outputs per
 //                 thread.
 #include <algorithm>
+#include <utility>
 
 #include "internal.h"
 
@@ -1120,7 +1121,7 @@ hef_status run_ortho(long long n, int K, T* V, long long ldv, double* R_out, int
 
 }  // namespace
 
-void ortho_allow_grid(bool on) { t_grid = on; }
+bool ortho_allow_grid(bool on) { return std::exchange(t_grid, on); }
 
 }  // namespace hef
 
