@@ -366,8 +366,8 @@ __global__ void __launch_bounds__(THREADS) k_chol_aug(const double* __restrict__
 //      lane = column) and so holds R11, its reciprocal diagonal and the kept
 //      flags, the same bits everywhere;
 //  (b) one thread per live column runs the panel's kPB eliminations down its
-//      column (the operations of k_chol_aug in its order) and publishes the
-//      panel rows; grid barrier;
+//      column (every element takes the operations of k_chol_aug in its order, so
+//      the two give the same bits) and publishes the panel rows; grid barrier;
 //  (c) every CTA reads the panel rows' left part, the multipliers, and updates
 //      the rows below in its columns; the owners publish the next diagonal
 //      block; grid barrier.
@@ -406,7 +406,9 @@ __global__ void __launch_bounds__(kGridThreads, 1)
   C* diag = static_cast<C*>(x.diag);
   for (int e = tid; e < ncol * K; e += kGridThreads) {
     const int q = b + nb * (e / K), i = e % K;
-    S[e] = q < K ? A[(size_t)q * K + i] : (q - K == i ? (C)1 : (C)0);  // A is symmetric
+    // row i of column q, as k_chol_aug reads it (G - c c^T / n is symmetric only
+    // up to rounding)
+    S[e] = q < K ? A[(size_t)i * K + q] : (q - K == i ? (C)1 : (C)0);
   }
   if (tid == 0) alive = 1;
   __syncthreads();
@@ -451,7 +453,7 @@ __global__ void __launch_bounds__(kGridThreads, 1)
           const C tn = __shfl_sync(0xffffffffu, thr_near, p);
           const bool kj = rf > (C)0 && d > tk;
           near_def |= (fast && kj && d <= tn) ? 1 : 0;
-          const C pv = kj ? rsqrt(d) : (C)0;
+          const C pv = kj ? pivot_rsqrt<C>(d) : (C)0;
           v[p] = kj ? v[p] * pv : (C)0;
 #pragma unroll
           for (int i = p + 1; i < kPB; ++i) {
