@@ -173,10 +173,18 @@ hef_status hef_incidence_check(const hef_incidence* inc, void* stream,
  *   (a copy on `stream`, which it synchronises), so that a test can plant an
  *   index that the checks must catch.  The regular build returns HEF_ERR_UNSUPPORTED and
  *   touches nothing; bad arguments give HEF_ERR_INVALID_ARG.
+ * hef_debug_inject: bounds-checked build only (else HEF_ERR_UNSUPPORTED): the
+ *   conditions `what` (a set of HEF_INJECT_*; 0: none) hold for later calls
+ *   from this thread, so that a test reaches the library's answer to them
+ *   without bringing them about on the GPU.
+ *   HEF_INJECT_REFUSED_GRID: cooperative launches are refused, as by a runtime
+ *   that grants the process fewer SMs than the device has.
  * ---------------------------------------------------------------------- */
+#define HEF_INJECT_REFUSED_GRID 1u
 int32_t hef_debug_checks(void);
 hef_status hef_debug_set_pin(const hef_incidence* inc, int64_t slot, int32_t value,
                              void* stream);
+hef_status hef_debug_inject(uint32_t what);
 
 hef_status hef_incidence_sizes(const hef_incidence* inc, int64_t* n,
                                int64_t* m, int64_t* P);

@@ -36,6 +36,7 @@ _SIGS = {
     "hef_abi_version": (c_i32, []),
     "hef_debug_checks": (c_i32, []),
     "hef_debug_set_pin": (c_i32, [c_p, c_i64, c_i32, c_p]),
+    "hef_debug_inject": (c_i32, [ctypes.c_uint32]),
     "hef_launch_count": (ctypes.c_uint64, []),
     "hef_trace_kernels": (c_i32, [ctypes.c_char_p]),
     "hef_trace_read": (c_i32, [c_i32, ctypes.c_char_p, ctypes.POINTER(c_i64),

@@ -162,4 +162,21 @@ extern "C" const char* hef_status_string(hef_status s) {
 
 extern "C" int32_t hef_abi_version(void) { return 1; }
 
+#if HEF_DEBUG
+namespace hef {
+static thread_local uint32_t t_inject = 0;
+bool injected(uint32_t what) { return (t_inject & what) != 0; }
+}  // namespace hef
+#endif
+
+extern "C" hef_status hef_debug_inject(uint32_t what) {
+#if HEF_DEBUG
+  hef::t_inject = what;
+  return HEF_OK;
+#else
+  (void)what;
+  return hef::set_error(HEF_ERR_UNSUPPORTED, "hef_debug_inject: not the bounds-checked build");
+#endif
+}
+
 extern "C" int32_t hef_debug_checks(void) { return HEF_DEBUG ? 1 : 0; }

@@ -113,12 +113,21 @@ inline cudaError_t launch_dependent_smem(void (*kernel)(KArgs...), unsigned grid
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// Whether a condition of hef_debug_inject is on for the calling thread (never
+// in the regular build).
+#if HEF_DEBUG
+bool injected(uint32_t what);
+#else
+constexpr bool injected(uint32_t) { return false; }
+#endif
+
 // Cooperative launch: the runtime starts the grid only with every CTA
 // resident at once (or refuses a grid that can never be), which is what a
 // kernel with grid-wide barriers needs when other work shares the GPU.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_cooperative_smem(void (*kernel)(KArgs...), unsigned grid, unsigned block,
                                            size_t smem, cudaStream_t st, Args... args) {
+  if (injected(HEF_INJECT_REFUSED_GRID)) return cudaErrorCooperativeLaunchTooLarge;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(block);

@@ -1041,9 +1041,10 @@ hef_status run_ortho(long long n, int K, T* V, long long ldv, double* R_out, int
       if (!want_R) o.R = nullptr;
       HEF_LAUNCH("k_gram_project", st, k_gram_project<<<stride_grid((long long)K * K, 2), kThreads, 0,
                                                          st>>>(w.G, w.c, K, (double)n, w.A64, w.A32));
-      // the factorisation by one CTA in shared memory, or by the grid where one
-      // SM's arithmetic (FP64) or shared memory (FP32) does not do and no other
-      // work of the caller's shares the GPU
+      // the factorisation by one CTA, or by the grid where one SM's arithmetic
+      // (FP64) or shared memory (FP32) does not do, no other work of the caller's
+      // shares the GPU and the runtime grants the grid (`taken`)
+      bool taken = false;
       auto on_grid = [&](auto zero, const auto* A, int fast) -> hef_status {
         using C = decltype(zero);
         // about two (FP64) or eight (FP32) live columns per CTA
@@ -1056,31 +1057,32 @@ hef_status run_ortho(long long n, int K, T* V, long long ldv, double* R_out, int
                    e = launch_cooperative_smem(k_chol_grid<C, T>, ctas, kGridThreads, smem, st,
                                                (const double*)w.G, (const double*)w.c, A, K, Kp,
                                                (double)n, tol, fast, x, o));
-        if (e != cudaSuccess) return set_error(HEF_ERR_CUDA, "k_chol_grid: %s", cudaGetErrorString(e));
+        taken = e == cudaSuccess;
+        if (!taken && e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorNotSupported)
+          return set_error(HEF_ERR_CUDA, "k_chol_grid: %s", cudaGetErrorString(e));
+        if (!taken) (void)cudaGetLastError();
         return HEF_OK;
       };
       if (fast_ok) {
         if (panels) {
           HEF_LAUNCH("k_chol_panels", st, k_chol_panels<T><<<1, kPanelThreads, panel_smem(K), st>>>(
                                               w.G, w.c, w.A32, K, Kp, (double)n, tol, o));
-        } else if (t_grid) {
-          hef_status s = on_grid(0.0f, (const float*)w.A32, 1);
-          if (s) return s;
         } else {
-          HEF_LAUNCH("k_chol_aug", st, k_chol_aug<float, T><<<1, 1024, 0, st>>>(
-                                           w.G, w.c, w.A32, K, Kp, (double)n, tol,
-                                           reinterpret_cast<float*>(w.Wg), 0, 1, 0, o));
+          if (t_grid)
+            if (hef_status s = on_grid(0.0f, (const float*)w.A32, 1)) return s;
+          if (!taken)
+            HEF_LAUNCH("k_chol_aug", st, k_chol_aug<float, T><<<1, 1024, 0, st>>>(
+                                             w.G, w.c, w.A32, K, Kp, (double)n, tol,
+                                             reinterpret_cast<float*>(w.Wg), 0, 1, 0, o));
         }
       }
       // exact FP64 path: always for the FP64 form, on demand for the FP32 form
-      if (!fast_ok && K >= kGridMinK && t_grid) {
-        hef_status s = on_grid(0.0, (const double*)w.A64, 0);
-        if (s) return s;
-      } else {
+      if (!fast_ok && K >= kGridMinK && t_grid)
+        if (hef_status s = on_grid(0.0, (const double*)w.A64, 0)) return s;
+      if (fast_ok || !taken)
         HEF_LAUNCH("k_chol_aug", st, k_chol_aug<double, T><<<1, 1024, 0, st>>>(
                                          w.G, w.c, w.A64, K, Kp, (double)n, tol, w.Wg, 0, 0,
                                          fast_ok ? 0 : 1, o));
-      }
     } else {
       HEF_CHECK_CUDA(cudaMemsetAsync(w.flag, 0, sizeof(int), st));  // flag[0] only
       HEF_LAUNCH("k_chol_series", st, k_chol_series<T><<<stride_grid((long long)Kp * Kp, 2),
