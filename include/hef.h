@@ -87,9 +87,10 @@ typedef int32_t hef_status;
 #define HEF_BAD_PIN 2u       /* a pin outside [0, n) */
 #define HEF_DUP_PIN 4u       /* a vertex repeated within one hyperedge */
 #define HEF_BAD_WEIGHT 8u    /* a weight that is not finite and > 0 */
-#define HEF_WAIT_TIMEOUT 16u /* a bounded grid-wide wait of the one-launch
-                                Krylov form expired (hef_incidence_check then
-                                returns HEF_ERR_TIMEOUT) */
+#define HEF_WAIT_TIMEOUT 16u /* a bounded wait of a kernel on this incidence
+                                (in a batched call also of its CholQR2)
+                                expired (hef_incidence_check then returns
+                                HEF_ERR_TIMEOUT) */
 #define HEF_BOUNDS 32u       /* HEF_DEBUG build: a kernel read a vertex or
                                 hyperedge index outside [0, n) or [0, m) from
                                 the incidence; the access was redirected to
@@ -179,8 +180,11 @@ hef_status hef_incidence_check(const hef_incidence* inc, void* stream,
  *   without bringing them about on the GPU.
  *   HEF_INJECT_REFUSED_GRID: cooperative launches are refused, as by a runtime
  *   that grants the process fewer SMs than the device has.
+ *   HEF_INJECT_EXPIRED_WAIT: hef_orthonormalize records an expired wait in its
+ *   last kernel.
  * ---------------------------------------------------------------------- */
 #define HEF_INJECT_REFUSED_GRID 1u
+#define HEF_INJECT_EXPIRED_WAIT 2u
 int32_t hef_debug_checks(void);
 hef_status hef_debug_set_pin(const hef_incidence* inc, int64_t slot, int32_t value,
                              void* stream);
@@ -289,7 +293,9 @@ hef_status hef_krylov_basis_ops(const hef_incidence* inc, int32_t k,
  * residual norms only down to about sqrt(machine epsilon)) is dropped: its Q
  * column is zero and scoring ignores it.
  * R_out (K x K double, row-major, nullable) receives R.  rank_out (one int32,
- * nullable) receives the number of kept columns.  K <= 512, n >= 1.
+ * nullable) receives the number of kept columns, or -1 when a bounded wait in
+ * one of the kernels ran out (Q and R are then not to be used; a batched call
+ * reports it as HEF_WAIT_TIMEOUT in the item's status).  K <= 512, n >= 1.
  * ---------------------------------------------------------------------- */
 size_t hef_orthonormalize_workspace_bytes(int64_t n, int32_t K, int32_t dtype);
 

@@ -9,6 +9,7 @@ is no other implementation.
 from __future__ import annotations
 
 import ctypes
+import math
 import os
 
 import torch
@@ -22,7 +23,8 @@ HEF_F64, HEF_F32, HEF_BF16 = 0, 1, 2
 HEF_REDUCE_MAX, HEF_REDUCE_SUM, HEF_REDUCE_EMBED = 0, 1, 2
 HEF_OPS_CLIQUE, HEF_OPS_STAR, HEF_OPS_BOTH = 1, 2, 3
 HEF_CLIQUE_HYPEREDGE, HEF_CLIQUE_PAPER = 0, 1
-HEF_ERR_INVALID_INPUT = -7
+HEF_ERR_TIMEOUT, HEF_ERR_INVALID_INPUT = -5, -7
+HEF_WAIT_TIMEOUT = 16
 
 _DTYPES = {HEF_F64: torch.float64, HEF_F32: torch.float32, HEF_BF16: torch.bfloat16}
 _CODES = {torch.float64: HEF_F64, torch.float32: HEF_F32, torch.bfloat16: HEF_BF16,
@@ -352,12 +354,16 @@ class HefResistance(torch.autograd.Function):
             V, tape = krylov_basis(inc, xc, xb, k, dtype), None
         Q, Rf, rank = orthonormalize(V, K, want_R=True)
         scores = edge_resistance(inc, Q, K)
-        ctx.state = (inc, k, xc, xb, Q, Rf, scores, tape, w.dtype)
-        return scores["R"].clone().to(w.dtype)
+        # without a synchronisation to raise at, a wait that ran out (rank -1)
+        # makes the scores and their gradients NaN
+        expired = rank < 0
+        ctx.state = (inc, k, xc, xb, Q, Rf, scores, tape, w.dtype, expired)
+        return scores["R"].clone().masked_fill_(expired, math.nan).to(w.dtype)
 
     @staticmethod
     def backward(ctx, gR):
-        inc, k, xc, xb, Q, Rf, scores, tape, wdt = ctx.state
+        inc, k, xc, xb, Q, Rf, scores, tape, wdt, expired = ctx.state
+        gR = gR.masked_fill(expired, math.nan)
         dw, dxc, dxb = edge_resistance_backward(inc, k, xc, xb, Q, Rf, scores, gR, tape=tape)
         ctx.state = None
         return dw.to(wdt), dxc, dxb, None, None, None, None, None, None, None
@@ -385,6 +391,13 @@ def orthonormalize(V, K, want_R=False, workspace=None, stream=None):
            L.hef_orthonormalize(n, K, code, _ptr(V), V.stride(0), _ptr(R), _ptr(rank),
                                 _ptr(workspace), workspace.numel(), _stream(stream)))
     return V, R, rank
+
+
+def check_rank(rank):
+    """Raise HefError if a bounded wait of hef_orthonormalize ran out
+    (synchronises)."""
+    if int(rank.item()) < 0:
+        raise HefError("hef_orthonormalize", HEF_ERR_TIMEOUT, "a tensor-core wait timed out")
 
 
 def edge_resistance(inc, Q, K, reduce=HEF_REDUCE_MAX, routing=True, workspace=None, out=None,
@@ -443,6 +456,7 @@ def hyperedge_resistance(n, eptr, pins, w, x0_clique, x0_star, k, dtype=torch.fl
     out = edge_resistance(inc, Q, K, reduce)
     if check:
         inc.check()
+        check_rank(rank)
     out.update(Q=Q[:, :K], rank=rank, incidence=inc)
     return out
 
@@ -517,8 +531,7 @@ class Pipeline:
         _check("hef_incidence_check",
                lib().hef_incidence_check(self.handle, _stream(stream), ctypes.byref(detail),
                                          ctypes.byref(where)))
-        if int(self.rank.item()) < 0:
-            raise HefError("hef_orthonormalize", -5, "a tensor-core wait timed out")
+        check_rank(self.rank)
 
     def capture(self, eptr, pins, w, x0_clique, x0_star):
         """Record one run on these input tensors as a CUDA graph; `replay()`
@@ -621,12 +634,17 @@ class Batch:
         return ns.value, list(sched), ms.value
 
     def check(self):
-        """Raise HefError if any item failed device validation."""
+        """Raise HefError if any item failed device validation or a bounded
+        wait of it ran out."""
         st = torch.stack([o["status"] for o in self.out]).cpu()
         bad = (st[:, 0] != 0).nonzero().flatten().tolist()
-        if bad:
-            raise HefError("hef_resistance_batched", HEF_ERR_INVALID_INPUT,
-                           f"items {bad} rejected by device validation")
+        if not bad:
+            return
+        if all(int(s) == HEF_WAIT_TIMEOUT for s in st[bad, 0]):
+            raise HefError("hef_resistance_batched", HEF_ERR_TIMEOUT,
+                           f"a bounded wait of items {bad} ran out")
+        raise HefError("hef_resistance_batched", HEF_ERR_INVALID_INPUT,
+                       f"items {bad} rejected by device validation")
 
     def capture(self):
         """Record one batched run as a CUDA graph; replay() reruns it."""
@@ -741,6 +759,7 @@ def multilevel(n, eptr, pins, w, starts, k, levels, dtype=torch.float32, quantil
         Q, _, rank = orthonormalize(V, K)
         sc = edge_resistance(inc, Q, K)
         inc.check()
+        check_rank(rank)
         lo = coarsen_level(inc, ep, pi, wl, sc["R"], eta, Q, K, sc["QH"], quantile=quantile)
         nc, nf, mc, pc = level_sizes(lo)
         of_orig = lo["final_cluster"][of_orig.long()]

@@ -134,7 +134,9 @@ hef_status run_item(const hef_batch_item& it, int k, int S, int dtype, int cliqu
                                      z.inc, st, &inc);
   if (s) return s;
   s = hef_krylov_basis(inc, k, S, dtype, it.x0_clique, it.x0_star, V, z.ldv, ws_kry, z.kry, st);
-  if (!s) s = hef_orthonormalize(it.n, K, dtype, V, z.ldv, nullptr, nullptr, ws_ortho, z.ortho, st);
+  if (!s)
+    s = orthonormalize(it.n, K, dtype, V, z.ldv, nullptr, nullptr, ws_ortho, z.ortho, inc->status,
+                       st);
   if (!s)
     s = hef_edge_resistance(inc, V, z.ldv, K, dtype, HEF_REDUCE_MAX, it.R_out, it.QH_out,
                             it.argvec, it.pmax, it.pmin, ws_score, z.score, st);
@@ -198,8 +200,8 @@ hef_status run_batch_one_launch(const hef_batch_item* items, int G, int k, int S
     cudaStream_t st = pool->s[sched[g]];
     if (!first && incs[g]) {
       void* V = p + z.inc + z.kry;
-      hef_status r = hef_orthonormalize(it.n, K, dtype, V, z.ldv, nullptr, nullptr,
-                                        p + z.inc + z.kry + z.V, z.ortho, st);
+      hef_status r = orthonormalize(it.n, K, dtype, V, z.ldv, nullptr, nullptr,
+                                    p + z.inc + z.kry + z.V, z.ortho, incs[g]->status, st);
       if (!r)
         r = hef_edge_resistance(incs[g], V, z.ldv, K, dtype, HEF_REDUCE_MAX, it.R_out, it.QH_out,
                                 it.argvec, it.pmax, it.pmin, p + z.inc + z.kry + z.V + z.ortho,

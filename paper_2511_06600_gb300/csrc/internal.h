@@ -216,6 +216,13 @@ bool krylov_allow_persistent(bool on);
 // whose launches could not all be resident.  Returns the setting it replaces.
 bool ortho_allow_grid(bool on);
 
+// hef_orthonormalize that also sets HEF_WAIT_TIMEOUT in `status` (an
+// incidence's status word; nullable) when a bounded wait ran out, for callers
+// that hand out no rank.
+hef_status orthonormalize(long long n, int K, int dtype, void* V, long long ldv, double* R_out,
+                          int32_t* rank_out, void* workspace, size_t workspace_bytes,
+                          unsigned int* status, cudaStream_t st);
+
 // The batched form's Krylov stage: per hypergraph, the starts on its own
 // stream (krylov_batch_start, workspace as for hef_krylov_basis); then all
 // k steps of every hypergraph in cooperative launches of up to 64

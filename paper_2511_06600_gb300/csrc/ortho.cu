@@ -815,13 +815,14 @@ __global__ void k_chol_series(const double* __restrict__ G, const double* __rest
   }
 }
 
-// rank = number of kept columns, or -1 when a tensor-core wait timed out
-// (flag[1]).
-__global__ void k_rank(const int* kept, int K, const int* flag, int* rank) {
+// rank = number of kept columns, or -1 when a bounded wait of either pass ran
+// out (flag[1]; so after the last apply), which then also goes into `status`.
+__global__ void k_rank(const int* kept, int K, const int* flag, int* rank, unsigned int* status) {
   if (threadIdx.x == 0) {
     int r = 0;
     for (int j = 0; j < K; ++j) r += kept[j];
     *rank = flag[1] ? -1 : r;
+    if (flag[1] && status) atomicOr(status, HEF_WAIT_TIMEOUT);
   }
 }
 
@@ -977,7 +978,7 @@ size_t carve_ortho(void* base, long long n, int K, int dtype, OrthoWs* w) {
 // the elimination; the Gram and the apply run on the tensor cores).
 template <typename T>
 hef_status run_ortho(long long n, int K, T* V, long long ldv, double* R_out, int* rank_out,
-                     const OrthoWs& w, cudaStream_t st, bool bf16 = false) {
+                     unsigned int* status, const OrthoWs& w, cudaStream_t st, bool bf16 = false) {
   const int Kp = round8(K);
   const size_t gram_smem = (size_t)kPR * Kp * sizeof(T);
   HEF_ENSURE_SMEM(k_gram<T>, (int)gram_smem);
@@ -1093,7 +1094,6 @@ hef_status run_ortho(long long n, int K, T* V, long long ldv, double* R_out, int
                      w.G, w.c, K, (double)n, w.A64, w.A32));
       HEF_LAUNCH("k_chol_aug", st, k_chol_aug<double, T><<<1, 1024, 0, st>>>(
                                        w.G, w.c, w.A64, K, Kp, (double)n, tol, w.Wg, 0, 0, 0, o));
-      HEF_LAUNCH("k_rank", st, k_rank<<<1, 32, 0, st>>>(w.kept, K, w.flag, w.rank));
     }
     HEF_CHECK_LAUNCH();
     if (sizeof(T) == 4 && apply_tc_supported(K)) {
@@ -1113,6 +1113,10 @@ hef_status run_ortho(long long n, int K, T* V, long long ldv, double* R_out, int
       HEF_CHECK_LAUNCH();
     }
   }
+  if (injected(HEF_INJECT_EXPIRED_WAIT))
+    HEF_CHECK_CUDA(cudaMemsetAsync(w.flag + 1, 1, sizeof(int), st));
+  HEF_LAUNCH("k_rank", st, k_rank<<<1, 32, 0, st>>>(w.kept, K, w.flag, w.rank, status));
+  HEF_CHECK_LAUNCH();
   if (R_out) {
     HEF_LAUNCH("k_trmm_upper", st, k_trmm_upper<<<stride_grid((long long)K * K, 4), kThreads, 0,
                                                   st>>>(w.R2, w.R1, K, R_out));
@@ -1127,21 +1131,9 @@ hef_status run_ortho(long long n, int K, T* V, long long ldv, double* R_out, int
 
 bool ortho_allow_grid(bool on) { return std::exchange(t_grid, on); }
 
-}  // namespace hef
-
-using namespace hef;
-
-extern "C" size_t hef_orthonormalize_workspace_bytes(int64_t n, int32_t K, int32_t dtype) {
-  if (n < 1 || K < 1 || K > 512 || (dtype != HEF_F64 && dtype != HEF_F32 && dtype != HEF_BF16))
-    return 0;
-  if (dtype == HEF_BF16 && !(gram_tc_supported(K) && apply_tc_supported(K))) return 0;
-  OrthoWs w;
-  return carve_ortho(nullptr, n, K, dtype, &w);
-}
-
-extern "C" hef_status hef_orthonormalize(int64_t n, int32_t K, int32_t dtype, void* V, int64_t ldv,
-                                         double* R_out, int32_t* rank_out, void* workspace,
-                                         size_t workspace_bytes, void* stream) {
+hef_status orthonormalize(long long n, int K, int dtype, void* V, long long ldv, double* R_out,
+                          int32_t* rank_out, void* workspace, size_t workspace_bytes,
+                          unsigned int* status, cudaStream_t st) {
   HEF_NVTX("hef_orthonormalize (Algorithm 1 step 4)");
   if (n < 1 || K < 1) return set_error(HEF_ERR_INVALID_ARG, "hef_orthonormalize: need n, K >= 1");
   if (K > 512) return set_error(HEF_ERR_UNSUPPORTED, "hef_orthonormalize: K must be <= 512");
@@ -1161,9 +1153,27 @@ extern "C" hef_status hef_orthonormalize(int64_t n, int32_t K, int32_t dtype, vo
   if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255) || workspace_bytes < need)
     return set_error(HEF_ERR_WORKSPACE,
                      "hef_orthonormalize: workspace needs %zu bytes (256-aligned)", need);
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (dtype == HEF_F64)
-    return run_ortho<double>(n, K, static_cast<double*>(V), ldv, R_out, rank_out, w, st);
-  return run_ortho<float>(n, K, static_cast<float*>(V), ldv, R_out, rank_out, w, st,
+    return run_ortho<double>(n, K, static_cast<double*>(V), ldv, R_out, rank_out, status, w, st);
+  return run_ortho<float>(n, K, static_cast<float*>(V), ldv, R_out, rank_out, status, w, st,
                           dtype == HEF_BF16);
+}
+
+}  // namespace hef
+
+using namespace hef;
+
+extern "C" size_t hef_orthonormalize_workspace_bytes(int64_t n, int32_t K, int32_t dtype) {
+  if (n < 1 || K < 1 || K > 512 || (dtype != HEF_F64 && dtype != HEF_F32 && dtype != HEF_BF16))
+    return 0;
+  if (dtype == HEF_BF16 && !(gram_tc_supported(K) && apply_tc_supported(K))) return 0;
+  OrthoWs w;
+  return carve_ortho(nullptr, n, K, dtype, &w);
+}
+
+extern "C" hef_status hef_orthonormalize(int64_t n, int32_t K, int32_t dtype, void* V, int64_t ldv,
+                                         double* R_out, int32_t* rank_out, void* workspace,
+                                         size_t workspace_bytes, void* stream) {
+  return orthonormalize(n, K, dtype, V, ldv, R_out, rank_out, workspace, workspace_bytes, nullptr,
+                        static_cast<cudaStream_t>(stream));
 }
