@@ -31,12 +31,14 @@
 //    2^-66 of the scale.  62 bits keep an entry's full 53 when it is down to
 //    2^-9 of its column's largest.  The mean is subtracted in the same
 //    integers, before the one rounding to FP64.
-// Entries that are not finite make their Gram row and column NaN (the column
-// is then dropped by the elimination, as with FP64 arithmetic) and their output
-// row NaN from the 64-column block on that reads them.
+// An entry that is not finite makes its column's mean and its Gram row and
+// column NaN (the column is then dropped by the elimination) and, as with FP64
+// arithmetic, whose products with the mean-free column are NaN in every row, all
+// rows of the output NaN from the 64-column block on that reads the column.
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <climits>
 
 #include "internal.h"
 #include "umma.cuh"
@@ -435,11 +437,13 @@ __host__ __device__ __forceinline__ size_t split_image(int J, int K) {
 // What an output column needs besides its digits: its values are
 // (sum - mean) 2^exp with the sum in units of level 5 and the mean of the
 // column (mu^T R^-1)_j split into an integer and a remainder of those units.
+// exp = kNanCol: a column that the output's block reads has no finite mean.
 struct SplitCol {
   long long mean;
   float mean_lo;
   int exp;
 };
+constexpr int kNanCol = INT_MIN;
 
 // The B operand's digits, laid out as the apply's stages take them: column j of
 // diag(2^E) R^-1 (the columns' scales moved into R^-1) on its own scale 2^F.
@@ -456,19 +460,22 @@ __global__ void k_split_rinv(const double* __restrict__ Rinv, const double* __re
   int F = 1;
   double m = 0.0;
   if (j < K) {
-    for (int i = lane; i <= j; i += 32) {
-      const double r = Rinv[(size_t)i * Kp + j];
+    bool nan = false;
+    for (int i = lane; i < min(kSpN * (J + 1), K); i += 32) {
+      const double a = mu[i], r = i <= j ? Rinv[(size_t)i * Kp + j] : 0.0;
       const int f = (__double2hiint(r) >> 20) & 0x7ff;
       if (r != 0.0) F = max(F, max(f, 1) + max(exps[i], 1));
-      m += mu[i] * r;
+      nan |= ((__double2hiint(a) >> 20) & 0x7ff) == kNotFinite || f == kNotFinite;
+      m += a * r;
     }
     F = __reduce_max_sync(0xffffffffu, F);
+    nan = __any_sync(0xffffffffu, nan);
     m = warp_sum(m);
     if (lane == 0) {
+      // |m| <= K 2^F 2^(-2 1022), as |mu_i| < 2^(E_i): |u| < 2^57
       const int e = F - 2 * 1022 - 12 - 7 * (kAExact - 1);
-      const double u = scalbn(m, -e), r = rint(u);
-      const bool fits = fabs(r) < 0x1p61;  // always, for a mean of the column's entries
-      cols[j] = SplitCol{fits ? (long long)r : 0ll, fits ? (float)(u - r) : 0.0f, e};
+      const double u = nan ? 0.0 : scalbn(m, -e), r = rint(u);
+      cols[j] = SplitCol{(long long)r, (float)(u - r), nan ? kNanCol : e};
     }
   }
   unsigned char* tile = image + split_image(J, K);
@@ -528,7 +535,6 @@ __global__ void __launch_bounds__(kSpThreads + 64, 1) k_apply_split(ApplySplitAr
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ uint64_t conv[2], full[2], empty[2], drained;
   __shared__ uint32_t tmem_slot;
-  __shared__ int bad[3][128];  // per block (mod 3): rows with an entry that is not finite
   __shared__ int colmax[512];
   constexpr uint32_t a_tile = 128u * 64u, a_stage = kAD * a_tile, b_stage = kAD * kSpN * 64u;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -538,7 +544,6 @@ __global__ void __launch_bounds__(kSpThreads + 64, 1) k_apply_split(ApplySplitAr
     mbar_init(&drained, kSpConv);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  for (int q = tid; q < 384; q += blockDim.x) bad[q >> 7][q & 127] = 0;
   for (int q = tid; q < 512; q += blockDim.x) colmax[q] = 0;
   tc_fence_before();
   __syncthreads();
@@ -548,7 +553,7 @@ __global__ void __launch_bounds__(kSpThreads + 64, 1) k_apply_split(ApplySplitAr
   const int nJ = (a.K + kSpN - 1) / kSpN;
   bool ok = true;
   uint32_t g = 0;    // stages so far; stage g uses buffer g % 2 for the (g / 2)-th time
-  uint32_t blk = 0;  // output blocks so far
+  uint32_t blk = 0;  // output blocks so far (MMA warp)
   if (warp == kSpConv + 1) {
     if (lane == 0) {  // B producer
       for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x)
@@ -637,21 +642,16 @@ __global__ void __launch_bounds__(kSpThreads + 64, 1) k_apply_split(ApplySplitAr
     };
     if ((int)blockIdx.x < ntiles) load(blockIdx.x, 0);
     for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-      for (int J = nJ - 1; J >= 0 && ok; --J, ++blk) {
+      for (int J = nJ - 1; J >= 0 && ok; --J) {
         const int nst = split_stages(J, a.K), Nj = split_width(J, a.K);
-        int* badrow = bad[blk % 3u];
         for (int st = 0; st < nst; ++st, ++g) {
           const int s = (int)(g & 1u);
           if (g >= 2) ok = mbar_wait(&empty[s], ((g >> 1) - 1) & 1u, kSpWait);
           if (!(ok = __all_sync(0xffffffffu, ok))) break;
-          bool broken = false;
+          // (an entry that is not finite has its column's scale: some digits,
+          // which reach outputs that are NaN by their kNanCol)
 #pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const bool inf = ((x[u] >> 52) & 0x7ff) == kNotFinite;
-            broken |= inf;
-            x[u] = biased_int<kAD>(inf ? 0ull : x[u], sc[u]);
-          }
-          if (broken) badrow[r] = 1;  // published to the drain by conv and the MMAs' commit
+          for (int u = 0; u < 8; ++u) x[u] = biased_int<kAD>(x[u], sc[u]);
           unsigned char* As = base + (size_t)s * (a_stage + b_stage) + my;
 #pragma unroll
           for (int j = 0; j < kAD; ++j) {
@@ -678,7 +678,6 @@ __global__ void __launch_bounds__(kSpThreads + 64, 1) k_apply_split(ApplySplitAr
         tc_fence_after();
         const int q4 = warp & 3;
         const long long row = (long long)tile * 128 + q4 * 32 + lane;
-        const bool nan_row = *reinterpret_cast<volatile int*>(badrow + q4 * 32 + lane) != 0;
         for (int c8 = warp >> 2; c8 < Nj / 8; c8 += kSpConv / 4) {
           long long h[8];  // levels 0..5; level l holds multiples of 2^(-7 l)
           float low[8];
@@ -705,9 +704,10 @@ __global__ void __launch_bounds__(kSpThreads + 64, 1) k_apply_split(ApplySplitAr
             v[u] = 0.0;
             if (jb + u < a.K) {
               const SplitCol col = a.cols[jb + u];
-              v[u] = to_double(h[u] - col.mean, low[u] * (float)(1ull << (7 * (kAExact - 1))) - col.mean_lo,
-                               col.exp);
-              if (nan_row) v[u] = __longlong_as_double(0x7ff8000000000000ll);
+              v[u] = col.exp == kNanCol
+                         ? __longlong_as_double(0x7ff8000000000000ll)
+                         : to_double(h[u] - col.mean,
+                                     low[u] * (float)(1ull << (7 * (kAExact - 1))) - col.mean_lo, col.exp);
             }
           }
           if (row < a.n) {
@@ -726,10 +726,6 @@ __global__ void __launch_bounds__(kSpThreads + 64, 1) k_apply_split(ApplySplitAr
             }
           }
         }
-        // every warp has drained the block before this one (it converted this
-        // block's stages after that), and none can reach the block that reuses
-        // those marks before this drain is over
-        if (warp < 4) bad[(blk + 2u) % 3u][warp * 32 + lane] = 0;
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&drained);
