@@ -10,9 +10,9 @@
 // 1.63 and 2.73 ms per pass with FP64 instructions, both bound by that pipe.
 // A product of two 53-bit numbers takes 43 (Gram, 8 digits) or 45 (apply, 9
 // digits) digit products, which the tensor cores do in a few per cent of that:
-// 0.19 and 0.23 ms now, bound by writing the digits.  Against 113-bit
-// arithmetic Q's error is 0.4 to 0.7 of the FP64 kernels' (1.0e-16 for 2.1e-16
-// per unit column on a Krylov basis of 9,999 x 64).
+// 0.19 and 0.27 ms now, bound by writing the digits.  Against 113-bit
+// arithmetic Q's error per unit column is 0.35 to 0.7 of the FP64 kernels'
+// (0.95e-16 for 2.1e-16 on a Krylov basis of 9,999 x 64).
 //
 // Digits.  A column of scale 2^E (|x| < 2^E for all its entries, from the
 // largest exponent in it) has x = 2^(E - 6) sum_j d_j 2^(-7j), |d_j| <= 64,
@@ -25,12 +25,25 @@
 //    leaving the level out costs 2^-57 (max / rms)^2 of a column's squared
 //    norm: 1.6e-14 where an entry is 48 times the rms).  A window leaves TMEM
 //    as two 64-bit integers per entry, which add up exactly over windows and
-//    CTAs, so the result does not depend on the grid.
+//    CTAs, so the result does not depend on the grid.  The error, 2^-56 of the
+//    columns' scales per row and so 2^-55 of their norms, is that of the
+//    triangular factor: it multiplies the rows of Q, and their differences,
+//    from the right.
 //  - apply: K <= 512 products per entry; levels 0..5 exact in six accumulators,
 //    levels 6..8 (weights 2^-42 and less) in a seventh, whose FP32 rounding is
-//    2^-66 of the scale.  62 bits keep an entry's full 53 when it is down to
-//    2^-9 of its column's largest.  The mean is subtracted in the same
-//    integers, before the one rounding to FP64.
+//    2^-66 of the scale.  Rows of V are scaled too, by the power of two that
+//    brings their largest entry (in units of its column's scale) to 2^0: a row is
+//    as accurate as any other, however small it is beside the columns' largest
+//    (62 bits of its largest entry; an error of 2^-60 of the row, where the
+//    rounding of R^-1 leaves 2^-53 of it).  The mean is subtracted in the same
+//    integers, before the one rounding to FP64.  Within a row, an output below
+//    2^-20 of its scale (the largest that |V| |R^-1| can be there), which would
+//    keep less than 40 bits, is formed again by FP64 multiply-adds, unless one of
+//    its products reaches that line by itself, so that FP64 would round at it as
+//    well.  On Krylov bases that is one output in 10^5 (at 2^-11 one in 100 and 80
+//    us at 50,851 x 160, for accuracy that the rounding of R^-1 hides).  Rows'
+//    scales, the exact means and this line took the apply there from 221 us per
+//    pass to 270.
 // An entry that is not finite makes its column's mean and its Gram row and
 // column NaN (the column is then dropped by the elimination) and, as with FP64
 // arithmetic, whose products with the mean-free column are NaN in every row, all
@@ -83,6 +96,8 @@ __device__ __forceinline__ uint64_t desc_k_sw64(uint32_t saddr) {
 __device__ __forceinline__ uint32_t sw64_offset(int row, int chunk) {
   return (uint32_t)(row * 64 + ((chunk ^ ((row >> 1) & 3)) * 16));
 }
+
+__device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 
 template <int D>
 struct Digits {
@@ -436,14 +451,21 @@ __host__ __device__ __forceinline__ size_t split_image(int J, int K) {
 
 // What an output column needs besides its digits: its values are
 // (sum - mean) 2^exp with the sum in units of level 5 and the mean of the
-// column (mu^T R^-1)_j split into an integer and a remainder of those units.
-// exp = kNanCol: a column that the output's block reads has no finite mean.
-struct SplitCol {
+// column m = (mu^T R^-1)_j split into an integer and a remainder of those units.
+// tag = 64 exp + the number of bits of |mean|, or kNanCol: a column that the
+// output's block reads has no finite mean.
+struct __align__(32) SplitCol {
   long long mean;
   float mean_lo;
-  int exp;
+  int tag;
+  double m;
 };
 constexpr int kNanCol = INT_MIN;
+constexpr int kColExp0 = -2 * 1022 - 12 - 7 * (kAExact - 1);  // exp of a column of R^-1 of scale 2^0
+// Columns below 2^(kTinyField - 1022): their squares underflow, so the
+// elimination has dropped them and R^-1 does not read them.
+constexpr int kTinyField = 256;
+constexpr int kWeakBits = 27;  // 2^-20 of the scale in units of level 5
 
 // The B operand's digits, laid out as the apply's stages take them: column j of
 // diag(2^E) R^-1 (the columns' scales moved into R^-1) on its own scale 2^F.
@@ -458,24 +480,40 @@ __global__ void k_split_rinv(const double* __restrict__ Rinv, const double* __re
   const int J = j / kSpN, jl = j % kSpN, Nj = split_width(J, K);
   const int nst = split_stages(J, K);
   int F = 1;
-  double m = 0.0;
   if (j < K) {
+    const int iend = min(kSpN * (J + 1), K);
     bool nan = false;
-    for (int i = lane; i < min(kSpN * (J + 1), K); i += 32) {
-      const double a = mu[i], r = i <= j ? Rinv[(size_t)i * Kp + j] : 0.0;
-      const int f = (__double2hiint(r) >> 20) & 0x7ff;
+    for (int i = lane; i < iend; i += 32) {
+      const double r = i <= j ? Rinv[(size_t)i * Kp + j] : 0.0;
+      const int f = exp_field(r);
       if (r != 0.0) F = max(F, max(f, 1) + max(exps[i], 1));
-      nan |= ((__double2hiint(a) >> 20) & 0x7ff) == kNotFinite || f == kNotFinite;
-      m += a * r;
+      nan |= exp_field(mu[i]) == kNotFinite || f == kNotFinite;
     }
     F = __reduce_max_sync(0xffffffffu, F);
     nan = __any_sync(0xffffffffu, nan);
-    m = warp_sum(m);
+    // m to more than FP64's precision: the outputs of refine_weak take the means
+    // off before their products, and must not differ from the others by a
+    // rounding of m.  |mu_i r| < 2^(F - 2 1022), so the parts of the products on
+    // the grid of `big` sum exactly, and the rest is 2^-43 of them.
+    const int fb = F - 2 * 1022 + 10 + 1023;
+    const double big = fb > 100 && fb < 2000 ? __hiloint2double(fb << 20, 0) : 0.0;
+    double hi = 0.0, lo = 0.0;
+    for (int i = lane; i <= j; i += 32) {
+      const double a = mu[i], r = Rinv[(size_t)i * Kp + j], p = __dmul_rn(a, r);
+      const double top = __dadd_rn(__dadd_rn(p, big), -big);
+      hi += top;
+      lo += (p - top) + fma(a, r, -p);
+    }
+    hi = warp_sum(hi);
+    lo = warp_sum(lo);
     if (lane == 0) {
       // |m| <= K 2^F 2^(-2 1022), as |mu_i| < 2^(E_i): |u| < 2^57
-      const int e = F - 2 * 1022 - 12 - 7 * (kAExact - 1);
-      const double u = nan ? 0.0 : scalbn(m, -e), r = rint(u);
-      cols[j] = SplitCol{(long long)r, (float)(u - r), nan ? kNanCol : e};
+      const int e = F + kColExp0;
+      const double u = nan ? 0.0 : scalbn(hi, -e), r = rint(u);
+      const double rest = nan ? 0.0 : (u - r) + scalbn(lo, -e), r2 = rint(rest);
+      const long long mean = (long long)r + (long long)r2;
+      cols[j] = SplitCol{mean, (float)(rest - r2),
+                         nan ? kNanCol : 64 * e + 64 - __clzll(llabs(mean)), hi + lo};
     }
   }
   unsigned char* tile = image + split_image(J, K);
@@ -502,6 +540,9 @@ struct ApplySplitArgs {
   const int* exps;
   const unsigned char* image;
   const SplitCol* cols;
+  const double* Rinv;  // row stride Kp
+  int Kp;
+  const double* mu;
   int* out_exps;  // largest exponent field of every output column, or null
   int* err;
 };
@@ -509,14 +550,99 @@ struct ApplySplitArgs {
 // (d + m) 2^e rounded to FP64, for an integer |d| < 2^62 and a small |m|
 // (in 62-bit integers: a 64-bit conversion and no FP64 arithmetic, which would
 // take four operations on a pipe of two per clock).
-__device__ __forceinline__ double to_double(long long d, float m, int e) {
+// `plain` becomes false when the result is outside FP64's normal range.
+__device__ __forceinline__ double scaled(long long d, float m, int e, bool& plain) {
   const unsigned long long mag = (unsigned long long)(d < 0 ? -d : d);
   const int s = min(max(__clzll((long long)mag) - 2, 0), 40);
   const long long t = (d << s) + __float2ll_rn(m * __int_as_float((127 + s) << 23));
   const double v = __ll2double_rn(t);
   const int hi = __double2hiint(v), f = ((hi >> 20) & 0x7ff) + e - s;
-  if (t != 0 && f >= 1 && f <= 2046) return __hiloint2double(hi + ((e - s) << 20), __double2loint(v));
-  return scalbn(v, e - s);
+  plain = plain && (t == 0 || (f >= 1 && f <= 2046));
+  return __hiloint2double(t == 0 ? 0 : hi + ((e - s) << 20), __double2loint(v));
+}
+// The same anywhere in FP64's range.
+__device__ __noinline__ double to_double(long long d, float m, int e) {
+  bool plain = true;
+  const double v = scaled(d, m, 0, plain);
+  return scalbn(v, e);
+}
+
+// The column's mean (mean + mean_lo) 2^s, in units of a row whose scale is 2^-s
+// of the columns', as an integer and a remainder, for s <= kPlainShift and a mean
+// of at most 61 - s bits: what almost every output takes.
+constexpr int kPlainShift = 21;
+__device__ __forceinline__ void shift_mean(const SplitCol& c, int s, long long& mean, float& rest) {
+  const float x = c.mean_lo * __int_as_float((127 + s) << 23);  // at most 2^20: rounded by a magic sum
+  const float t = x + 12582912.0f;
+  mean = (c.mean << s) + (__float_as_int(t) - 0x4b400000);
+  rest = x - (t - 12582912.0f);
+}
+
+// An output (sum h + l in units of a row of scale 2^rs, minus the mean) without
+// those limits; weak: below the line of refine_weak.
+__device__ __noinline__ double odd_output(const SplitCol& c, long long h, float l, int rs, bool& weak) {
+  if (c.tag == kNanCol) return __longlong_as_double(0x7ff8000000000000ll);
+  const int s = -rs, e = c.tag >> 6, bits = c.tag & 63;
+  const float x = scalbnf(c.mean_lo, s);
+  // a mean of 2^5 times what the row's own sum can be, or more
+  if (!(fabsf(x) < 0x1p60f) || (bits > 0 && bits + s > 61)) return to_double(h, l, e + rs) - c.m;
+  const long long i = __float2ll_rn(x), d = h - (bits > 0 ? c.mean << s : 0) - i;
+  weak = llabs(d) < (1ll << kWeakBits);
+  return to_double(d, l - (x - __ll2float_rn(i)), e + rs);
+}
+
+// The mark of a row of zeros (isolated vertices: a few per cent of a netlist's),
+// whose scale is 2^0.
+constexpr int kZeroRow = 1;
+
+// Outputs of a warp's 32 rows (lane = row, from row0) and columns jb + u whose
+// bit u is set in `weak`: formed again in FP64 where no product of theirs
+// reaches the line (see the head of the file); `shift`: the row's scale.  Eight
+// lanes per output, four outputs of different rows at a time.
+__device__ __forceinline__ void refine_weak(const ApplySplitArgs& a, long long row0, int jb, int shift,
+                                            unsigned weak, double (&v)[8]) {
+  const int lane = threadIdx.x & 31, grp = lane >> 3, sub = lane & 7;
+  while (const unsigned todo = __ballot_sync(0xffffffffu, weak != 0)) {
+    unsigned t = todo;
+    for (int q = 0; q < grp; ++q) t &= t - 1;
+    const bool have = t != 0;
+    const int src = have ? __ffs(t) - 1 : 0;
+    const int j = jb + max(__ffs(__shfl_sync(0xffffffffu, weak, src)) - 1, 0);
+    const double* vr = a.V + (row0 + src) * a.ldv;
+    const double* rc = a.Rinv + j;
+    int top = 0;  // a product is at least 2^(top - 2047)
+    if (have) {
+#pragma unroll 4
+      for (int i = sub; i <= j; i += 8) {
+        const int fv = exp_field(vr[i]), fr = exp_field(rc[(size_t)i * a.Kp]);
+        if (fv >= exp_field(a.mu[i]) + 2 && fr > 0) top = max(top, fv + fr);
+      }
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, o));
+    const int rs = __shfl_sync(0xffffffffu, shift, src);
+    const int redo = have && top < (a.cols[j].tag >> 6) + rs + kWeakBits + 2047;
+    double s = 0.0;
+    if (__any_sync(0xffffffffu, redo)) {
+      if (redo) {
+#pragma unroll 4
+        for (int i = sub; i <= j; i += 8) s = fma(vr[i] - a.mu[i], rc[(size_t)i * a.Kp], s);
+      }
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    }
+    // the first four rows that had one take theirs
+    const int rank = __popc(todo & ((1u << lane) - 1u));
+    const double got = __shfl_sync(0xffffffffu, s, (rank & 3) * 8);
+    const int take = __shfl_sync(0xffffffffu, redo, (rank & 3) * 8);
+    if (weak != 0 && rank < 4) {
+      const int u0 = __ffs(weak) - 1;
+      weak &= weak - 1;
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (take && u == u0) v[u] = got;
+    }
+  }
 }
 
 // Q = (V - 1 mu^T) R^-1 = V R^-1 - 1 (mu^T R^-1) in place, a tile of 128 rows
@@ -533,18 +659,24 @@ __global__ void __launch_bounds__(kSpThreads + 64, 1) k_apply_split(ApplySplitAr
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  __shared__ uint64_t conv[2], full[2], empty[2], drained;
+  __shared__ uint64_t conv[2], full[2], empty[2], drained, rows[4];
   __shared__ uint32_t tmem_slot;
-  __shared__ int colmax[512];
+  __shared__ int colmax[512], shifts[2][128];  // row scales of this and the next tile
+  __shared__ __align__(16) int scales[512];    // exponent fields of the columns' scales
   constexpr uint32_t a_tile = 128u * 64u, a_stage = kAD * a_tile, b_stage = kAD * kSpN * 64u;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (warp == 0) tmem_alloc(&tmem_slot, 512);
   if (tid == 0) {
     for (int q = 0; q < 2; ++q) mbar_init(&conv[q], kSpConv), mbar_init(&full[q], 1), mbar_init(&empty[q], 1);
     mbar_init(&drained, kSpConv);
+    for (int q = 0; q < 4; ++q) mbar_init(&rows[q], kSpConv / 4);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  for (int q = tid; q < 512; q += blockDim.x) colmax[q] = 0;
+  for (int q = tid; q < 512; q += blockDim.x) {
+    const int e = q < a.K ? a.exps[q] : 0;
+    scales[q] = e >= kTinyField ? e : 2 * 0x7ff + 64;  // all digits 0, whatever the row's scale
+    colmax[q] = 0;
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -623,6 +755,39 @@ __global__ void __launch_bounds__(kSpThreads + 64, 1) k_apply_split(ApplySplitAr
     const uint32_t my = sw64_offset(r, chunk);
     uint64_t x[8];
     int sc[8];
+    uint32_t stored = 0;  // rounds of the drain so far
+    int shift = 0;        // scale of this thread's row: its largest entry beside its column's
+    auto row_shift = [&](int tile) {
+      const long long row = (long long)tile * 128 + r;
+      int top = -0x7ff;
+      uint64_t any = 0;
+      if (a.K <= kSpHalf) {  // the whole row is in the four threads' stage
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          any |= x[u];
+          top = max(top, max((int)(x[u] >> 52) & 0x7ff, 1) - sc[u]);
+        }
+      } else if (row < a.n) {  // 16 bytes of it at a time, eight loads in flight
+        const double2* p = reinterpret_cast<const double2*>(a.V + row * a.ldv);
+        const int np = a.K / 2;
+#pragma unroll 8
+        for (int c = chunk; c < np; c += 4) {
+          const double2 x = p[c];
+          const int2 e = *reinterpret_cast<const int2*>(scales + 2 * c);
+          any |= (uint64_t)__double_as_longlong(x.x) | (uint64_t)__double_as_longlong(x.y);
+          top = max(top, max(max(exp_field(x.x), 1) - e.x, max(exp_field(x.y), 1) - e.y));
+        }
+        if ((a.K & 1) && chunk == 0) {
+          const double x = a.V[row * a.ldv + a.K - 1];
+          any |= (uint64_t)__double_as_longlong(x);
+          top = max(top, max(exp_field(x), 1) - scales[a.K - 1]);
+        }
+      }
+      if (any << 1 == 0) top = -0x7ff;
+      top = max(top, __shfl_xor_sync(0xffffffffu, top, 1));
+      top = max(top, __shfl_xor_sync(0xffffffffu, top, 2));
+      return top == -0x7ff ? kZeroRow : top;
+    };
     auto load = [&](int tile, int st) {
       const long long row = (long long)tile * 128 + r;
       const int c = st * kSpHalf + 8 * chunk;
@@ -638,10 +803,18 @@ __global__ void __launch_bounds__(kSpThreads + 64, 1) k_apply_split(ApplySplitAr
         x[u + 1] = (uint64_t)__double_as_longlong(v.y);
       }
 #pragma unroll
-      for (int u = 0; u < 8; ++u) sc[u] = c + u < a.K ? max(__ldg(a.exps + c + u), 1) : 1;
+      for (int u = 0; u < 8; u += 4) {
+        const int4 e = *reinterpret_cast<const int4*>(scales + c + u);
+        sc[u] = e.x, sc[u + 1] = e.y, sc[u + 2] = e.z, sc[u + 3] = e.w;
+      }
     };
     if ((int)blockIdx.x < ntiles) load(blockIdx.x, 0);
-    for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+    int buf = 0;
+    for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, buf ^= 1) {
+      // read by the drains, after the MMAs of stages that follow this
+      shift = row_shift(tile);
+      if (chunk == 0) shifts[buf][r] = shift;
+      shift = min(shift, 0);
       for (int J = nJ - 1; J >= 0 && ok; --J) {
         const int nst = split_stages(J, a.K), Nj = split_width(J, a.K);
         for (int st = 0; st < nst; ++st, ++g) {
@@ -651,7 +824,7 @@ __global__ void __launch_bounds__(kSpThreads + 64, 1) k_apply_split(ApplySplitAr
           // (an entry that is not finite has its column's scale: some digits,
           // which reach outputs that are NaN by their kNanCol)
 #pragma unroll
-          for (int u = 0; u < 8; ++u) x[u] = biased_int<kAD>(x[u], sc[u]);
+          for (int u = 0; u < 8; ++u) x[u] = biased_int<kAD>(x[u], sc[u] + shift);
           unsigned char* As = base + (size_t)s * (a_stage + b_stage) + my;
 #pragma unroll
           for (int j = 0; j < kAD; ++j) {
@@ -678,38 +851,72 @@ __global__ void __launch_bounds__(kSpThreads + 64, 1) k_apply_split(ApplySplitAr
         tc_fence_after();
         const int q4 = warp & 3;
         const long long row = (long long)tile * 128 + q4 * 32 + lane;
-        for (int c8 = warp >> 2; c8 < Nj / 8; c8 += kSpConv / 4) {
-          long long h[8];  // levels 0..5; level l holds multiples of 2^(-7 l)
-          float low[8];
-          const uint32_t at = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(c8 * 8);
-#pragma unroll
-          for (int half = 0; half < 2; ++half) {  // within the registers of 18 warps
-            float L[3][8];
-#pragma unroll
-            for (int l = 0; l < 3; ++l) tmem_ld8(at + (uint32_t)((3 * half + l) * Nj), L[l]);
-            if (half) tmem_ld8(at + (uint32_t)(kAExact * Nj), low);
-            tmem_wait_ld();
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-              if (!half) h[u] = 0;
-#pragma unroll
-              for (int l = 0; l < 3; ++l)
-                h[u] = h[u] * 128 + __float2int_rn(L[l][u] * (float)(1ull << (7 * (3 * half + l))));
-            }
-          }
+        const int mark = shifts[buf][q4 * 32 + lane], rs = min(mark, 0);
+        const bool zero_row = mark == kZeroRow;
+        // rounds of four column octets, one per warp of these rows, from the last
+        // to the first; a round is stored when all four have read what they need
+        // of the rows (columns up to their own)
+        for (int round = (Nj / 8 - 1) / 4; round >= 0; --round) {
+          const int c8 = 4 * round + (warp >> 2);
+          const bool on = c8 < Nj / 8;  // warp-uniform
           const int jb = J * kSpN + c8 * 8;
           double v[8];
+          if (on) {
+            long long h[8];  // levels 0..5; level l holds multiples of 2^(-7 l)
+            float low[8];    // levels 6..8
+            const uint32_t at = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(c8 * 8);
 #pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            v[u] = 0.0;
-            if (jb + u < a.K) {
-              const SplitCol col = a.cols[jb + u];
-              v[u] = col.exp == kNanCol
-                         ? __longlong_as_double(0x7ff8000000000000ll)
-                         : to_double(h[u] - col.mean,
-                                     low[u] * (float)(1ull << (7 * (kAExact - 1))) - col.mean_lo, col.exp);
+            for (int half = 0; half < 2; ++half) {  // within the registers of 18 warps
+              float L[3][8];
+#pragma unroll
+              for (int l = 0; l < 3; ++l) tmem_ld8(at + (uint32_t)((3 * half + l) * Nj), L[l]);
+              if (half) tmem_ld8(at + (uint32_t)(kAExact * Nj), low);
+              tmem_wait_ld();
+#pragma unroll
+              for (int u = 0; u < 8; ++u) {
+                if (!half) h[u] = 0;
+#pragma unroll
+                for (int l = 0; l < 3; ++l)
+                  h[u] = h[u] * 128 + __float2int_rn(L[l][u] * (float)(1ull << (7 * (3 * half + l))));
+              }
             }
+            unsigned weak = 0, odd = 0;
+            const int s = min(-rs, kPlainShift);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+              low[u] *= (float)(1ull << (7 * (kAExact - 1)));
+              v[u] = 0.0;
+              if (jb + u < a.K) {
+                const SplitCol col = a.cols[jb + u];
+                long long mean;
+                float rest;
+                shift_mean(col, s, mean, rest);
+                const long long d = h[u] - mean;
+                bool plain = -rs <= kPlainShift && (col.tag & 63) + s <= 61 && col.tag != kNanCol;
+                v[u] = scaled(d, low[u] - rest, (col.tag >> 6) + rs, plain);
+                // (not where R^-1's column is zero)
+                if (((unsigned long long)(d + (1ll << kWeakBits)) >> (kWeakBits + 1)) == 0 &&
+                    col.tag >= 64 * (2 + kColExp0))
+                  weak |= 1u << u;
+                if (!plain) odd |= 1u << u;
+              }
+            }
+            if (__any_sync(0xffffffffu, odd != 0)) {
+#pragma unroll
+              for (int u = 0; u < 8; ++u)
+                if ((odd >> u) & 1u) {
+                  bool w = false;
+                  v[u] = odd_output(a.cols[jb + u], h[u], low[u], rs, w);
+                  weak = (weak & ~(1u << u)) | ((w ? 1u : 0u) << u);
+                }
+            }
+            refine_weak(a, row - lane, jb, rs, row < a.n && !zero_row ? weak : 0u, v);
           }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&rows[q4]);
+          ok = mbar_wait(&rows[q4], stored++ & 1u, kSpWait);
+          if (!(ok = __all_sync(0xffffffffu, ok))) break;
+          if (!on) continue;
           if (row < a.n) {
             double* dst = a.V + row * a.ldv + jb;
 #pragma unroll
@@ -726,6 +933,7 @@ __global__ void __launch_bounds__(kSpThreads + 64, 1) k_apply_split(ApplySplitAr
             }
           }
         }
+        if (!ok) break;
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&drained);
@@ -818,6 +1026,9 @@ hef_status apply_split(double* V, long long ldv, long long n, int K, const doubl
   a.exps = exps;
   a.image = w.image;
   a.cols = reinterpret_cast<const SplitCol*>(w.cols);
+  a.Rinv = Rinv;
+  a.Kp = Kp;
+  a.mu = mu;
   a.out_exps = out_exps;
   a.err = err;
   const size_t smem = 1024 + 2 * (size_t)kAD * (128 + kSpN) * 64;
