@@ -293,11 +293,11 @@ hef_status hef_krylov_basis_ops(const hef_incidence* inc, int32_t k,
  * residual norms only down to about sqrt(machine epsilon)) is dropped: its Q
  * column is zero and scoring ignores it.
  * Precision of HEF_F64: R is that of a Gram matrix with an error of 2^-55 of
- * the columns' norms (before the mean is taken off; up to 2^27 rows), and Q = (V
+ * the columns' norms (before the mean is taken off), and Q = (V
  * - 1 mu^T) R^-1 has a further error of 2^-60 of each row (its largest entry in
  * units of its column's); entries below 2^-20 of their row are formed by FP64
- * multiply-adds.  Q is at least as close to the exact factor as by FP64
- * arithmetic throughout, and so are differences of rows.
+ * multiply-adds.  Measured, Q is closer to the exact factor than by FP64
+ * arithmetic, which is what more than 2^27 rows take.
  * R_out (K x K double, row-major, nullable) receives R.  rank_out (one int32,
  * nullable) receives the number of kept columns, or -1 when a bounded wait in
  * one of the kernels ran out (Q and R are then not to be used; a batched call

@@ -254,7 +254,7 @@ hef_status apply_tc(void* V, bool bf16, long long ldv, long long n, int K, const
                     int Kp, const float* mu, float* scratch, int* err, cudaStream_t st);
 
 // FP64 Gram and apply by error-free splitting on the tensor cores
-// (ortho_split.cu), for n <= 2^28 rows and K <= 512: exps holds two rows of K
+// (ortho_split.cu), for n <= 2^27 rows and K <= 512: exps holds two rows of K
 // exponent fields (the basis as given, then the first pass's output).
 struct SplitWs {
   long long* hi;
@@ -263,7 +263,10 @@ struct SplitWs {
   unsigned char* cols;   // per output column: mean and scale
   unsigned char* image;  // digits of R^-1
 };
-inline bool split_supported(long long n) { return n <= (1ll << 28); }
+// |lo| of the Gram's sums grows by less than 2^35.4 per row (levels 4 to 8: at
+// most 5, 6, 7 and 8 + 7 products of digits up to 64, in units of level 7, times
+// 2^21, 2^14, 2^7 and 1), and must stay below 2^63.
+inline bool split_supported(long long n) { return n <= (1ll << 27); }
 size_t carve_split(Carver& cv, long long n, int K, SplitWs* w);
 hef_status split_col_exps(const double* V, long long ldv, long long n, int K, const SplitWs& w,
                           cudaStream_t st);

@@ -8,7 +8,7 @@
 //
 // Kernels (the Gram and the apply run on the tensor cores: ortho_tc.cu for the
 // FP32 and BF16 forms up to K = 511, ortho_split.cu for the FP64 form up to
-// 2^28 rows; k_gram and k_apply serve what those do not take)
+// 2^27 rows; k_gram and k_apply serve what those do not take)
 //  k_gram         partial Gram of a row chunk: thread = 8x8 block of the
 //                 upper triangle, FP32 (or FP64) accumulation per chunk, FP64
 //                 partials; k_gram_reduce sums chunks in a fixed order.
