@@ -235,7 +235,8 @@ hef_status hef_krylov_basis(const hef_incidence* inc, int32_t k, int32_t S,
 /* Launch form of the Krylov calls made from the calling host thread
  * (a library setting; the paper has no counterpart).  on = 1 (default): all
  * k steps run as one cooperative launch of at most one CTA per SM (one per
- * 128 of the n + m rows).  Each CTA owns a
+ * 128 of the n + m rows; in FP32 below 32,768 rows one per 512, or 384 for S >=
+ * 8, which leaves SMs to calls on other streams).  Each CTA owns a
  * balanced range of vertices and hyperedges, keeps their index lists in
  * shared memory across the steps, and meets the others at bounded grid-wide
  * barriers that carry the Lanczos reductions (a barrier that waits too long

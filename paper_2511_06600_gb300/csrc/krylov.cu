@@ -953,12 +953,25 @@ __global__ void __launch_bounds__(kThreads) k_archive_last(IncView g, KView<T> k
 constexpr unsigned int kBarIters = 1u << 21;  // bounded barrier wait (polls of an L2 line: about 1 s)
 constexpr int kCapItems = 4096;               // vertices / hyperedges cached per CTA
 // Rows (n + m) per CTA from which the persistent form takes another CTA, up to
-// one per SM.  Measured from 1 to 152 CTAs: the time of small hypergraphs is
-// flat from about one CTA per 128 rows on (2,048 vertices in FP64, S = 1: 216 us
-// with 32 or 152 CTAs; 8,827 in FP32, S = 4: 302 to 311 us from 64 to 152), and
-// CTAs that gain nothing are left to other streams.  The three launches per
-// step take 377 and 539 us there, so the persistent form runs at every size.
+// one per SM.  The three launches per step are slower at every size and S (k = 10,
+// 2,025 to 84,000 vertices: FP64 S = 1 374 to 659 us for 214 to 385, S = 4 575 to
+// 1268 for 372 to 914; FP32 S = 4 270 to 415 for 165 to 232, S = 8 296 to 509 for
+// 197 to 354; FP32 S = 16 435 for 385 at 2,025 and 910 for 959 at 84,000), but
+// those of several streams overlap, where a cooperative grid waits until all its
+// CTAs fit.  So CTAs that gain little are left to other streams below
+// kSharedRows in FP32: 8,827 vertices, S = 4, one call 168 us with 128 rows per
+// CTA, 174 with 512 (200 with 1024); eight streams of whole calls 379 us a call
+// with 128 rows, 170 with 512, 236 with launches per step.  S >= 8, whose CTAs
+// have half the threads: 208 us with 128 rows, 212 with 384, 239 with 512.  In
+// FP64 a CTA's arithmetic counts: S = 2 286, 294, 344 us with 128, 256, 512 rows,
+// and eight streams take 340 us a call with 128 for 478 with launches per step.
 constexpr long long kPersistentRows = 128;
+constexpr long long kSharedRows = 32768;
+template <typename T, int S>
+long long rows_per_cta(long long rows) {
+  if (sizeof(T) == 8 || rows >= kSharedRows) return kPersistentRows;
+  return S <= 4 ? 512 : 384;
+}
 constexpr int kCapList = 12288;               // incidences / pins cached per CTA
 constexpr int kPartSlots = 9;                 // reduction slots per start (see part_buffer)
 
@@ -1439,9 +1452,9 @@ hef_status run_krylov_s(const hef_incidence* inc, int k, const double* x0c, cons
   // (the batched form); if the runtime refuses the grid, three launches per
   // step run instead
   if (persistent && n > 0 && m > 0) {
-    const int ctas = t_force_oversized
-                         ? num_sms()
-                         : (int)std::min<long long>(num_sms(), (n + m + kPersistentRows - 1) / kPersistentRows);
+    const long long rpc = rows_per_cta<T, S>(n + m);
+    const int ctas =
+        t_force_oversized ? num_sms() : (int)std::min<long long>(num_sms(), (n + m + rpc - 1) / rpc);
     constexpr int NT = pers_threads<T, S>();
     constexpr size_t kSmemLimit = 227 * 1024;  // per-CTA opt-in limit of the sm_100 family
     // list capacities: 1.25 times the average range (the balanced ranges
