@@ -371,8 +371,8 @@ constexpr int kBulkThreads = 512;  // warp 0 produces, warps 1..15 consume
 constexpr int kConsumers = kBulkThreads / 32 - 1;
 constexpr int kGroupWin = 8;    // windows per prefetch group of the producer
 constexpr int kMetaEdges = 128;  // hyperedge offsets / weights staged per window
-constexpr int kFlushWin = 32;    // windows per working-type partial sum of a consumer lane: about ten
-                                 // hyperedges of a group, then four groups, before FP64 takes over
+constexpr int kFlushWin = 8;     // windows per working-type partial sum: about three hyperedges of a
+                                 // group and four groups, before FP64 takes over
 constexpr int kEdgeLanes = 8;    // lanes per hyperedge
 constexpr int kGroupPins = 12;   // longer hyperedges take the whole warp
 constexpr int kPartChunks = 6;   // 16-byte chunks per lane at most: 768 bytes of a row per part
