@@ -13,10 +13,14 @@
 //                 upper triangle, FP32 (or FP64) accumulation per chunk, FP64
 //                 partials; k_gram_reduce sums chunks in a fixed order.
 //  k_chol_aug     one CTA: Gauss elimination of [G | I] -> [R | R^-T] (the
-//                 inverse comes out of the same K pivot steps).  FP32 in
-//                 shared memory for the FP32 form's first pass; FP64 (global
-//                 scratch) as the exact path: the FP64 form's first pass, and
-//                 the fallback when a fast pass reports near rank deficiency.
+//                 inverse comes out of the same K pivot steps) in global
+//                 scratch.  FP64 as the exact path: the FP64 form's first pass,
+//                 and the fallback when a fast pass reports near rank
+//                 deficiency; FP32 where the grid is not to be had beyond K = 160.
+//  k_chol_panels  the FP32 form's first pass up to K = 160: the same in one CTA's
+//                 shared memory.
+//  k_chol_grid    the same over the whole grid: FP64 from K = 48, FP32 beyond
+//                 K = 160.
 //  k_chol_series  second pass: R2 = I + X1, R2^-1 = I - X1 (X1 = upper part of
 //                 E with halved diagonal); exact to O(|E|^2); falls back to the
 //                 exact path when |E| is not small.
@@ -201,21 +205,19 @@ __device__ __forceinline__ double pivot_rsqrt<double>(double d) {
 // Gauss elimination of [A | I] with A = G - c c^T / n: after pivot j, row j
 // holds R[j][j..K) on the left and (R^-T)[j][0..j] on the right.  Columns
 // whose pivot is <= tol * G_jj are dropped (their rows stay zero).
-// C: arithmetic type; W: the K x 2K work matrix (shared or global memory).
+// C: arithmetic type; W: the K x 2K work matrix (global memory, L2-resident).
 // fast = 1: report (flag) any kept pivot <= 1e-4 G_jj instead of trusting
 // it.  fast = 0: exact path; runs only when `flag` is set unless `always`.
-template <typename C, typename T, int THREADS = 1024>
-__global__ void __launch_bounds__(THREADS) k_chol_aug(const double* __restrict__ G,
+template <typename C, typename T>
+__global__ void __launch_bounds__(1024) k_chol_aug(const double* __restrict__ G,
                                                    const double* __restrict__ c,
                                                    const C* __restrict__ Aproj, int K, int Kp,
-                                                   double n, double tol, C* Wg, int use_smem,
-                                                   int fast, int always, CholOut o) {
-  extern __shared__ unsigned char sm_raw[];
+                                                   double n, double tol, C* W, int fast, int always,
+                                                   CholOut o) {
   __shared__ C ref[512], thr_keep[512], thr_near[512];
   __shared__ int pk[kPB];  // kept flags of the current panel
   __shared__ int near_def;
   if (!fast && !always && o.flag[0] == 0) return;
-  C* W = use_smem ? reinterpret_cast<C*>(sm_raw) : Wg;
   const int W2 = 2 * K;
   for (int i = (int)(threadIdx.x >> 5); i < K; i += (int)(blockDim.x >> 5)) {
     C* row = W + (size_t)i * W2;
@@ -282,38 +284,23 @@ __global__ void __launch_bounds__(THREADS) k_chol_aug(const double* __restrict__
 #pragma unroll
     for (int p = 0; p < kPB; ++p) npb += (j0 + p < jend) ? 1 : 0;
     if (sizeof(C) == 4 && (K & 3) == 0 && (jend & 3) == 0) {
-      // FP32: four columns per lane (16-byte shared-memory accesses), kUR rows
-      // per warp at a time, so that a lane has 4 kUR independent FMA chains
-      // (one row with 1024 threads, whose 64 registers hold no more)
-      constexpr int kUR = THREADS >= 1024 ? 1 : 4;
-      for (int i0 = jend + wid * kUR; i0 < K; i0 += nw * kUR) {
-        float rj[kUR][kPB];
+      // FP32: four columns per lane (16-byte accesses)
+      for (int i = jend + wid; i < K; i += nw) {
+        float rj[kPB];
 #pragma unroll
-        for (int r = 0; r < kUR; ++r)
-#pragma unroll
-          for (int p = 0; p < kPB; ++p)
-            rj[r][p] = (i0 + r < K && p < npb && pk[p]) ? (float)W[(size_t)(j0 + p) * W2 + i0 + r] : 0.0f;
+        for (int p = 0; p < kPB; ++p)
+          rj[p] = (p < npb && pk[p]) ? (float)W[(size_t)(j0 + p) * W2 + i] : 0.0f;
+        float4* rowi = reinterpret_cast<float4*>(reinterpret_cast<float*>(W + (size_t)i * W2) + jend);
         for (int v = lane; v < K / 4; v += 32) {
-          float4 acc[kUR];
-#pragma unroll
-          for (int r = 0; r < kUR; ++r)
-            acc[r] = i0 + r < K ? reinterpret_cast<const float4*>(
-                                      reinterpret_cast<const float*>(W + (size_t)(i0 + r) * W2) + jend)[v]
-                                : make_float4(0.f, 0.f, 0.f, 0.f);
+          float4 acc = rowi[v];
 #pragma unroll
           for (int p = 0; p < kPB; ++p) {
             const float4 b =
                 reinterpret_cast<const float4*>(reinterpret_cast<float*>(W + (size_t)(j0 + p) * W2) + jend)[v];
-#pragma unroll
-            for (int r = 0; r < kUR; ++r) {
-              acc[r].x -= rj[r][p] * b.x, acc[r].y -= rj[r][p] * b.y;
-              acc[r].z -= rj[r][p] * b.z, acc[r].w -= rj[r][p] * b.w;
-            }
+            acc.x -= rj[p] * b.x, acc.y -= rj[p] * b.y;
+            acc.z -= rj[p] * b.z, acc.w -= rj[p] * b.w;
           }
-#pragma unroll
-          for (int r = 0; r < kUR; ++r)
-            if (i0 + r < K)
-              reinterpret_cast<float4*>(reinterpret_cast<float*>(W + (size_t)(i0 + r) * W2) + jend)[v] = acc[r];
+          rowi[v] = acc;
         }
       }
     } else {
@@ -1074,7 +1061,7 @@ hef_status run_ortho(long long n, int K, T* V, long long ldv, double* R_out, int
           if (!taken)
             HEF_LAUNCH("k_chol_aug", st, k_chol_aug<float, T><<<1, 1024, 0, st>>>(
                                              w.G, w.c, w.A32, K, Kp, (double)n, tol,
-                                             reinterpret_cast<float*>(w.Wg), 0, 1, 0, o));
+                                             reinterpret_cast<float*>(w.Wg), 1, 0, o));
         }
       }
       // exact FP64 path: always for the FP64 form, on demand for the FP32 form
@@ -1082,7 +1069,7 @@ hef_status run_ortho(long long n, int K, T* V, long long ldv, double* R_out, int
         if (hef_status s = on_grid(0.0, (const double*)w.A64, 0)) return s;
       if (fast_ok || !taken)
         HEF_LAUNCH("k_chol_aug", st, k_chol_aug<double, T><<<1, 1024, 0, st>>>(
-                                         w.G, w.c, w.A64, K, Kp, (double)n, tol, w.Wg, 0, 0,
+                                         w.G, w.c, w.A64, K, Kp, (double)n, tol, w.Wg, 0,
                                          fast_ok ? 0 : 1, o));
     } else {
       HEF_CHECK_CUDA(cudaMemsetAsync(w.flag, 0, sizeof(int), st));  // flag[0] only
@@ -1093,7 +1080,7 @@ hef_status run_ortho(long long n, int K, T* V, long long ldv, double* R_out, int
                  k_gram_project<<<stride_grid((long long)K * K, 2), kThreads, 0, st>>>(
                      w.G, w.c, K, (double)n, w.A64, w.A32));
       HEF_LAUNCH("k_chol_aug", st, k_chol_aug<double, T><<<1, 1024, 0, st>>>(
-                                       w.G, w.c, w.A64, K, Kp, (double)n, tol, w.Wg, 0, 0, 0, o));
+                                       w.G, w.c, w.A64, K, Kp, (double)n, tol, w.Wg, 0, 0, o));
     }
     HEF_CHECK_LAUNCH();
     if (sizeof(T) == 4 && apply_tc_supported(K)) {
