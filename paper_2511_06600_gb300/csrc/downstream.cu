@@ -252,7 +252,7 @@ __device__ __forceinline__ double qval(const T* Q, long long ldq, long long row,
 // exact, and the corrected quotient is off by less than 2^-104 of itself before
 // its rounding, while a quotient by k that is no rounding boundary lies at
 // least 2^-54 / k away from one.  Three FP64 operations (one when k is a power
-// of two) instead of a division's eight and its special cases; tiny and
+// of two) instead of a division's sequence and its special cases; tiny and
 // non-finite values take the division.
 __device__ __forceinline__ double div_by_int(double a, double k, double rk, bool pow2) {
   const int f = (__double2hiint(a) >> 20) & 0x7ff;
@@ -339,9 +339,10 @@ __global__ void __launch_bounds__(kThreads)
 // scored by max over columns of (Q[p,i] - mu_c[i])^2 / Q_H[i]; the smallest
 // score wins, ties to the smallest cluster id.
 //
-// The scores are FP64 (round to nearest), and FP64 division is what bound this
-// kernel (two DFMA per clock and SM): K divisions per candidate pin, 5.68 ms at
-// 210,000 vertices, K = 160; 0.46 ms now.  A candidate is now bounded in FP32 first: with
+// The scores are FP64 (round to nearest), and FP64 division would bound this
+// kernel (two DFMA per clock and SM): with K divisions per candidate pin it takes
+// 5.68 ms at 210,000 vertices, K = 160, as it is 0.46 ms.  A candidate is bounded
+// in FP32 first: with
 // q, m the FP32 values of Q[p,i] and mu_c[i] (rounded and truncated), |Q - mu|
 // lies within err = 1.5 2^-23 (|q| + |m|) of |q - m|, which gives [lb_i, ub_i] around each
 // column's ratio and [max lb, max ub] around the score (the constants below
@@ -350,10 +351,10 @@ __global__ void __launch_bounds__(kThreads)
 // only the columns with ub_i >= max lb can hold the maximum, and only those
 // are formed in FP64: one or two divisions for a few candidates per vertex,
 // with the same result bit for bit.  Columns are held NC per lane, so a
-// candidate costs one FP32 row of gathers.  What remained was the chain of
-// dependent loads from a vertex to its candidates' rows, walked once per
-// hyperedge: the lanes now take the pins of up to 32 hyperedges together, 32
-// pins at a time, which walks it once for most vertices.
+// candidate costs one FP32 row of gathers.  What remains is the chain of
+// dependent loads from a vertex to its candidates' rows: the lanes take the pins
+// of up to 32 hyperedges together, 32 pins at a time, which walks it once for
+// most vertices instead of once per hyperedge.
 // CTAs of two warps: a CTA keeps its registers until its slowest vertex is done,
 // and about half the vertices have nothing to do.
 constexpr int kSeedThreads = 64;
@@ -548,17 +549,16 @@ __global__ void k_final_ids(int n, const int32_t* __restrict__ cluster, const in
 }
 
 // Distinct clusters of a hyperedge, first occurrences in pin order: with
-// `out`, written there; returns their count.  The start of this work had one
-// thread per hyperedge compare every pin with all earlier ones through global
-// memory: the longest hyperedge's thread set the time (a 400-pin net makes
-// 80,000 dependent two-step gathers; 2.7 ms per kernel at 200,000 nets).  Now
-// a lane keeps up to kRegPins clusters in registers, which covers 96 % of a
-// netlist's hyperedges, and longer ones are taken by their warp, 32 pins at a
-// time: equal clusters within a round meet by a warp match, earlier rounds by
-// a hash table in shared memory, so that the work is linear in the pins.
-// Hyperedges too long for the table compare their rounds with all earlier
-// ones from registers instead.  Both kernels are then bound by the two gathers
-// per pin: 2747 -> 23 us (fill) and 2736 -> 21 us (count) at 200,000 nets.
+// `out`, written there; returns their count.  A thread per hyperedge that
+// compares every pin with all earlier ones is as slow as the longest hyperedge
+// (a 400-pin net makes 80,000 dependent two-step gathers).  Here a lane keeps up
+// to kRegPins clusters in registers, which covers 96 % of a netlist's
+// hyperedges, and longer ones are taken by their warp, 32 pins at a time: equal
+// clusters within a round meet by a warp match, earlier rounds by a hash table
+// in shared memory, so that the work is linear in the pins.  Hyperedges too long
+// for the table compare their rounds with all earlier ones from registers
+// instead.  Both kernels are then bound by the two gathers per pin: 2747 -> 23 us
+// (fill) and 2736 -> 21 us (count) at 200,000 nets.
 constexpr int kRegPins = 8;
 constexpr int kHashSlots = 1024;             // per warp; at most half full
 constexpr int kHashPins = kHashSlots / 2;    // longer hyperedges skip the table

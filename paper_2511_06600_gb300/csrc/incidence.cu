@@ -446,7 +446,7 @@ constexpr int kRecips = 64;
 // product is within two ulps, its residual exact, and the corrected quotient
 // rounds correctly (a quotient by k that is no rounding boundary lies at least
 // 2^-54 / k away from one, the correction's error is below 2^-104).  Three FP64
-// operations, one for powers of two, instead of a division's eight and its
+// operations, one for powers of two, instead of a division's sequence and its
 // special cases.
 __device__ __forceinline__ double div_small(double a, int k, const double2* recip) {
   const int f = (__double2hiint(a) >> 20) & 0x7ff;

@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(1024) k_chol_aug(const double* __restrict__ G,
 //      the rows below in its columns; the owners publish the next diagonal
 //      block; grid barrier.
 // The diagonal block's serial chain, the columns' and two barriers, 28 us (FP64)
-// or 19 us (FP32) per panel, are what remains: FP64 K = 160 763 -> 287 us, FP32
+// or 19 us (FP32) per panel, are what remains: FP64 K = 160 763 -> 289 us, FP32
 // K = 384 1210 -> 453 us.
 constexpr int kGridThreads = 256;
 constexpr int kGridMinK = 48;  // FP64: below, one CTA takes less than the barriers

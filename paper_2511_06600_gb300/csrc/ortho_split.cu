@@ -386,7 +386,8 @@ __global__ void __launch_bounds__(kSpThreads + 32, 1) k_gram_split(GramSplitArgs
 }
 
 // G (K x K, FP64) and c (K): the chunks' integers summed (exactly, so in any
-// order), then one rounding to FP64 and the columns' scales.
+// order), then rounded to FP64 (each half, where it passes 2^53, and their sum)
+// and put on the columns' scales.
 __global__ void __launch_bounds__(256) k_gram_split_reduce(const long long* __restrict__ hi,
                                                            const long long* __restrict__ lo, int K,
                                                            int Kc, int nchunk,

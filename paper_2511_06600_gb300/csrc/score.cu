@@ -229,8 +229,8 @@ __global__ void __launch_bounds__(256) k_score_big1(IncView g, const QT* __restr
 
 // This CTA's share of the large hyperedges' partials of column col: rows
 // blockIdx.x, blockIdx.x + gridDim.x, ... (after k_score_big1 has completed).
-// Every CTA adds its own rows to its partial: the last CTA used to add all of
-// them, one dependent load after another, 32 us at the end of a 130 us pass.
+// Every CTA adds its own rows to its partial: all of them in the last CTA, one
+// dependent load after another, take 25 to 30 us at the end of the pass.
 __device__ __forceinline__ double big_share(const double* __restrict__ bpart, int nbpart, int K,
                                             int col) {
   double s = 0.0;
@@ -358,14 +358,13 @@ __global__ void __launch_bounds__(256) k_score_pass1(IncView g, const QT* __rest
 // and still takes part in the reduction.
 //
 // What bounds it: 4 kWinSlots bytes of rows per slot through L2 and the
-// consumers' issue.  Scalar lanes took 20 loads, 20 stores and their addresses
-// per hyperedge and column block; chunks take a quarter.  Parts keep at least
-// four stages in flight where a row is long: with two (K = 384 in FP32, 160 in
-// FP64) every copy was waited for.  Rows whose pitch has no room for the 32-byte
-// rounding, and rows of more than 256 values, used one bulk copy per row.
-// 200,000 nets, K = 160, FP32: 132 -> 117 us (of it 25 us in the last CTA's sum
-// of k_score_big1's partials); 105,001 nets, K = 100: 131 -> 66; 1.3 M nets,
-// K = 384: 2016 -> 1166; FP64, 53,393 nets, K = 160: 309 -> 121 (comparisons).
+// consumers' issue.  Lanes of one value take 20 loads, 20 stores and their
+// addresses per hyperedge and column block; chunks take a quarter.  Parts keep at
+// least four stages in flight where a row is long: with two (K = 384 in FP32, 160
+// in FP64) every copy is waited for.  With chunks, parts, gathers for every width
+// (else one bulk copy per row past 256 values) and big_share together: 200,000
+// nets, K = 160, FP32 132 -> 117 us; 105,001 nets, K = 100 131 -> 66; 1.3 M nets,
+// K = 384 2016 -> 1166; FP64, 53,393 nets, K = 160 309 -> 121 (comparisons).
 static_assert(kBigEdge <= kWinSlots, "a scored hyperedge must end within the next window");
 constexpr int kBulkThreads = 512;  // warp 0 produces, warps 1..15 consume
 constexpr int kConsumers = kBulkThreads / 32 - 1;
