@@ -245,7 +245,8 @@ hef_status hef_krylov_basis(const hef_incidence* inc, int32_t k, int32_t S,
  * (work on other streams delays it rather than starving a barrier); if it
  * refuses the grid, or with on = 0, three launches per step run instead.
  * Both forms give the same results up to the order of floating-point sums.
- * hef_resistance_batched always uses the per-step form.  on = 2 exercises
+ * hef_resistance_batched has a setting of its own (hef_set_batch_krylov_form)
+ * and leaves this one as it was.  on = 2 exercises
  * the timeout path: the persistent form is launched (plainly) with twice the
  * CTAs that can be resident, so its first barrier cannot complete; the
  * launch ends after the wait limit with HEF_WAIT_TIMEOUT set and later calls
